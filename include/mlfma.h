@@ -276,8 +276,9 @@ mlfma_status mlfma_tune(mlfma_plan_t plan, int64_t B, int x_is_complex, int prec
  *   [3 + 44 + l]  translation at level l: 1 two columns per thread; 2..6 one
  *                 column with 1, 2, 4, 8, 16 lanes per output; 7 / 8 one warp
  *                 per (child, sample) with 2 / 1 columns per lane; 9 / 10 / 11
- *                 four columns per thread and the children four at a time,
- *                 64 / 32 / 16 columns per CTA (FP32 only)
+ *                 four columns per thread and the children four at a time:
+ *                 the variant the built-in choice takes, the next entry's
+ *                 sources requested ahead, not requested ahead (FP32 only)
  * Columns per CTA are powers of two (1, 2, 4, 8, 16).  mlfma_tune_set
  * returns MLFMA_EINVAL, and pins nothing, for B outside 1..max_batch, an
  * unknown prec or a value outside the sets above; a listed shape that does

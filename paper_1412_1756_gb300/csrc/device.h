@@ -267,10 +267,11 @@ cudaError_t launch_down_win(const DevLevel<float> &P, const DevLevel<float> &Ch,
 cudaError_t prime_win_kernels();
 
 // Translation of FP32 fields grouped by parent, four columns per thread and
-// the children four at a time (translate_quad.cu), NB = 16, 32 or 64
-// columns per CTA.  cudaErrorInvalidConfiguration, with nothing launched,
-// when the level's tables or shared memory do not fit the kernel.
-cudaError_t launch_translate_quad(const DevLevel<float> &lv, int B, int Bs, int acc, int nb, cudaStream_t s);
+// the children four at a time (translate_quad.cu).  variant 32: the next
+// entry's sources requested ahead, 16: not, else the built-in choice.
+// cudaErrorInvalidConfiguration, with nothing launched, when the level's
+// tables or shared memory do not fit the kernel.
+cudaError_t launch_translate_quad(const DevLevel<float> &lv, int B, int Bs, int acc, int variant, cudaStream_t s);
 cudaError_t prime_translate_quad();
 
 // Reception of FP32 fields, two columns per thread with the field tile

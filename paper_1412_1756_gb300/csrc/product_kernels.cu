@@ -1655,13 +1655,13 @@ cudaError_t launch_translate_es(const DevLevel<R> &Lv, int B, int Bs, int acc, c
 template <class R>
 cudaError_t launch_translate(const DevLevel<R> &Lv, int B, int Bs, int acc, cudaStream_t s, int choice = 0)
 {
-    if (choice >= 9 && choice <= 11) {   // four columns per thread, 64 / 32 / 16 columns per CTA
+    if (choice >= 9 && choice <= 11) {   // four columns per thread; 10 / 11 pin one of its two variants
         if constexpr (sizeof(R) == 4) return launch_translate_quad(Lv, B, Bs, acc, 64 >> (choice - 9), s);
         else return cudaErrorInvalidConfiguration;
     }
     if constexpr (sizeof(R) == 4) {
         if (choice == 0 && B >= 16) {   // built-in for wide batches: four columns per thread
-            const cudaError_t e = launch_translate_quad(Lv, B, Bs, acc, B >= 64 ? 64 : (B >= 32 ? 32 : 16), s);
+            const cudaError_t e = launch_translate_quad(Lv, B, Bs, acc, 0, s);
             if (e != cudaErrorInvalidConfiguration) return e;
         }
     }
