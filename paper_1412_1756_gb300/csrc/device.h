@@ -283,4 +283,23 @@ cudaError_t launch_receive_pairs(const ProductArgs<float> &a, int Bs, int nb, cu
 cudaError_t launch_radiate_quads(const ProductArgs<float> &a, int Bs, cudaStream_t s);
 cudaError_t prime_receive_pairs();
 
+// Radiation and reception by register tiles (leaf_tile.cu), any number of
+// columns; Bs as the other leaf launchers.  cudaErrorInvalidConfiguration,
+// with nothing launched, when the largest leaf box does not fit shared memory.
+template <class R>
+cudaError_t launch_radiate_tile(const ProductArgs<R> &a, int Bs, cudaStream_t s);
+template <class R>
+cudaError_t launch_receive_tile(const ProductArgs<R> &a, int Bs, cudaStream_t s);
+template <class R>
+cudaError_t prime_leaf_tile();
+
+// Near field by register tiles of four rows (near_tile.cu), any number of
+// columns.  cudaErrorInvalidConfiguration, with nothing launched, when a
+// chunk of the largest strip exceeds kNearTileSmem bytes of shared memory.
+constexpr int kNearTileSmem = 200 * 1024;
+template <class R>
+cudaError_t launch_near_tile(const ProductArgs<R> &a, cudaStream_t s);
+template <class R>
+cudaError_t prime_near_tile();
+
 }  // namespace mlfma

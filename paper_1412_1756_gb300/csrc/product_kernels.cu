@@ -1404,6 +1404,9 @@ cudaError_t launch_near_wide(const ProductArgs<R> &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// Leaf boxes too few to give every SM two CTAs at one per box and 16 columns.
+bool few_boxes(int64_t boxes, int B) { return boxes * ((B + 15) / 16) < 2 * 152; }
+
 template <class R>
 cudaError_t launch_near(const ProductArgs<R> &a, cudaStream_t s, int choice = 0)
 {
@@ -1412,6 +1415,12 @@ cudaError_t launch_near(const ProductArgs<R> &a, cudaStream_t s, int choice = 0)
     if (choice == 1) return wide_ok ? launch_near_wide<R, 8>(a, s) : cudaErrorInvalidConfiguration;
     if (choice == 2) return wide_ok ? launch_near_wide<R, 16>(a, s) : cudaErrorInvalidConfiguration;
     if (choice == 3) return a.B >= 16 ? launch_near_bt<R, 16>(a, s) : cudaErrorInvalidConfiguration;
+    // register tiles: FP32 from two columns up; FP64, which its arithmetic bounds, where the tree has too few
+    // leaf boxes to fill the GPU with one CTA per box (near_tile.cu has the figures of both sides)
+    if (sizeof(R) == 4 ? a.B >= 2 : (a.B >= 4 && few_boxes(a.nr.nleaf, a.B))) {
+        const cudaError_t e = launch_near_tile<R>(a, s);
+        if (e != cudaErrorInvalidConfiguration) return e;
+    }
     // wide path: all columns per strip pass (B a multiple of 16 bytes of R and BPT)
     if (a.B >= 32 && wide_ok) {
         if (a.B <= 256) return launch_near_wide<R, 8>(a, s);   // 8 columns x rows per thread; row tiles of 256 / (B/8)
@@ -1450,10 +1459,15 @@ cudaError_t launch_radiate(const ProductArgs<R> &a, int Bs, cudaStream_t s, int 
         else return cudaErrorInvalidConfiguration;
     }
     if constexpr (sizeof(R) == 4) {
-        if (choice == 0 && a.B >= 32) {   // built-in for wide batches
+        if (choice == 0 && a.B % 64 == 0) {   // whole 64-column chunks
             const cudaError_t e = launch_radiate_quads(a, Bs, s);
             if (e != cudaErrorInvalidConfiguration) return e;
         }
+    }
+    // register tiles that follow the columns (leaf_tile.cu has the figures of both sides)
+    if (choice == 0 && (sizeof(R) == 4 ? a.B >= 2 : (a.B >= 4 && few_boxes(Lf.nbox, a.B)))) {
+        const cudaError_t e = launch_radiate_tile<R>(a, Bs, s);
+        if (e != cudaErrorInvalidConfiguration) return e;
     }
     if (choice >= 2 && choice <= 4) {
         const int nb = choice == 2 ? 32 : choice == 3 ? 16 : 8;
@@ -1521,8 +1535,14 @@ cudaError_t launch_receive(const ProductArgs<R> &a, int Bs, cudaStream_t s, int 
         if constexpr (sizeof(R) == 4) return launch_receive_pairs(a, Bs, 64 >> (choice - 4), s);
         else return cudaErrorInvalidConfiguration;
     }
-    if constexpr (sizeof(R) == 4)
-        if (choice == 0 && a.B >= 32) return launch_receive_pairs(a, Bs, 32, s);   // built-in for wide batches
+    if (choice == 0) {
+        // register tiles that follow the columns (leaf_tile.cu has the figures of both sides); one full chunk of 16
+        // is left to the 16-column kernel
+        if (sizeof(R) == 8 ? a.B >= 3 : (a.B >= 2 && a.B != 16)) {
+            const cudaError_t e = launch_receive_tile<R>(a, Bs, s);
+            if (e != cudaErrorInvalidConfiguration) return e;
+        }
+    }
     if (choice == 1) return a.B >= 32 ? launch_receive_tiled<R, 32>(a, Bs, s) : cudaErrorInvalidConfiguration;
     if (choice == 2) return a.B >= 16 ? launch_receive_tiled<R, 16>(a, Bs, s) : cudaErrorInvalidConfiguration;
     if (choice == 3) return a.B >= 8 ? launch_receive_tiled<R, 8>(a, Bs, s) : cudaErrorInvalidConfiguration;
@@ -1821,6 +1841,8 @@ cudaError_t prime_kernels()
     ALLOW_UP(1); ALLOW_UP(2); ALLOW_UP(4); ALLOW_UP(8); ALLOW_UP(16);
 #undef ALLOW_UP
 #undef ALLOW
+    if ((e = prime_near_tile<R>()) != cudaSuccess) return e;
+    if ((e = prime_leaf_tile<R>()) != cudaSuccess) return e;
     if (sizeof(R) == 4) {
         if ((e = prime_win_kernels()) != cudaSuccess) return e;
         if ((e = prime_receive_pairs()) != cudaSuccess) return e;
