@@ -257,7 +257,8 @@ cudaError_t launch_down_umma(const DevLevel<float> &P, const DevLevel<float> &Ch
                              cudaStream_t s);
 
 // Windowed CUDA-core interpolation and anterpolation of FP32 fields
-// (window_interp.cu), NB = 4, 8 or 16 columns per CTA.
+// (window_interp.cu); nb as the tune values less 300, 0: the built-in shape
+// for the level and the columns.
 // cudaErrorInvalidConfiguration, with nothing launched, when the level has
 // no windowed tables or does not fit the kernels.
 cudaError_t launch_up_win(const DevLevel<float> &P, const DevLevel<float> &Ch, int B, int Bs, int acc, int nb,

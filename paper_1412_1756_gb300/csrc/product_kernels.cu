@@ -1624,13 +1624,14 @@ cudaError_t launch_up(const DevLevel<R> &P, const DevLevel<R> &Ch, int B, int Bs
     using C = typename Cx<R>::T;
     if (nb_choice > 300) {   // 304, 308, 316 windowed FP32 kernel with 4 / 8 / 16 columns per CTA; 404, 408 the
                              // same with 4 / 8 columns and registers for one more CTA per SM; 704, 708, 716
-                             // with the children that differ only in z sharing one phi step
+                             // with the children that differ only in z sharing one phi step; 754, 758 those with
+                             // registers for one more CTA per SM
         if constexpr (sizeof(R) == 4) return launch_up_win(P, Ch, B, Bs, acc, nb_choice - 300, s);
         else return cudaErrorInvalidConfiguration;
     }
     if constexpr (sizeof(R) == 4) {
-        if (nb_choice == 0 && B >= 16) {   // built-in for wide batches: windowed with z pairs, 8 columns per CTA
-            const cudaError_t e = launch_up_win(P, Ch, B, Bs, acc, 408, s);
+        if (nb_choice == 0 && B >= 2) {   // built-in: windowed, with z pairs where the level has the split shift
+            const cudaError_t e = launch_up_win(P, Ch, B, Bs, acc, 0, s);
             if (e != cudaErrorInvalidConfiguration) return e;
         }
     }
@@ -1778,15 +1779,14 @@ cudaError_t launch_down(const DevLevel<R> &P, const DevLevel<R> &Ch, int B, int 
     if (nb_choice > 300) {   // 304, 308, 316 windowed FP32 kernel with 4 / 8 / 16 columns per CTA; 404, 408 the
                              // same with 4 / 8 columns and registers for one more CTA per SM; 504, 508 one
                              // CTA per parent (its field loaded once for all children), 4 / 8 columns; 804, 808
-                             // per pair of children that differ only in z (one phi step for both)
+                             // per pair of children that differ only in z (one phi step for both), 854 the 4-column
+                             // one with 512 threads
         if constexpr (sizeof(R) == 4) return launch_down_win(P, Ch, B, Bs, nb_choice - 300, s);
         else return cudaErrorInvalidConfiguration;
     }
     if constexpr (sizeof(R) == 4) {
-        if (nb_choice == 0 && B >= 16) {   // built-in for wide batches: windowed with z pairs, 8 then 4 columns
-            cudaError_t e = launch_down_win(P, Ch, B, Bs, 508, s);
-            if (e != cudaErrorInvalidConfiguration) return e;
-            e = launch_down_win(P, Ch, B, Bs, 504, s);
+        if (nb_choice == 0 && B >= 3) {   // built-in: windowed, with z pairs where the level has the split shift
+            const cudaError_t e = launch_down_win(P, Ch, B, Bs, 0, s);
             if (e != cudaErrorInvalidConfiguration) return e;
         }
     }

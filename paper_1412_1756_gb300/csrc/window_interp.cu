@@ -15,7 +15,8 @@
 // (reversed order, the column at phi + pi), the direct rows and the other
 // pole's reflected rows (three segments).  No table is read from global
 // memory inside the stencil loops: the coefficients and window starts are
-// copied into shared memory once per CTA.
+// copied into shared memory once per CTA.  The products with the z factors
+// spell out their fused operations, so that every instantiation rounds alike.
 #include "device.h"
 
 #include <algorithm>
@@ -296,8 +297,8 @@ __device__ __forceinline__ void down_prefetch(float4 (&xin)[PF], const float2 *d
 // conj(shift_xy) * conj(gam(theta)); the parent is shifted by the pair's
 // common conj(shift_xy) and anterpolated in phi once, and each child's theta
 // step runs on U with its rows scaled by that child's conj(gam).
-template <int NB, int MINB, bool PAIR = false>
-__global__ void __launch_bounds__(256, MINB) k_down_win(DevLevel<float> P, DevLevel<float> Ch, int B, int Bs)
+template <int NB, int MINB, bool PAIR = false, int NT = 256>
+__global__ void __launch_bounds__(NT, MINB) k_down_win(DevLevel<float> P, DevLevel<float> Ch, int B, int Bs)
 {
     constexpr int NCP = NB / 2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -346,7 +347,7 @@ __global__ void __launch_bounds__(256, MINB) k_down_win(DevLevel<float> P, DevLe
     __syncthreads();
     down_phi<NB>(H4, U4, cph, sph, wp, ntp, nphp, nphc);
     __syncthreads();
-    constexpr int PF = MINB >= 4 ? 1 : kPF;   // fewer prefetch registers for the tighter budget
+    constexpr int PF = (MINB >= 4 || NT > 256) ? 1 : kPF;   // fewer prefetch registers for the tighter budget
     const int nch = pair ? 2 : 1;
     for (int k = 0; k < nch; ++k) {
         const int c = k ? cb : ca;
@@ -361,13 +362,13 @@ __global__ void __launch_bounds__(256, MINB) k_down_win(DevLevel<float> P, DevLe
                 float2 f = make_float2(a.x, -a.y);
                 if (k) {
                     const float2 b = gb[t];   // a * conj(b)
-                    f = make_float2(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
+                    f = make_float2(fmaf(a.x, b.x, __fmul_rn(a.y, b.y)), fmaf(a.y, b.x, -__fmul_rn(a.x, b.y)));
                 }
                 float4 *row = U4 + (size_t)t * up * NCP;
                 for (int i = lane; i < nphc * NCP; i += 32) {
                     const float4 u = row[i];
-                    row[i] = make_float4(f.x * u.x - f.y * u.y, f.x * u.y + f.y * u.x, f.x * u.z - f.y * u.w,
-                                         f.x * u.w + f.y * u.z);
+                    row[i] = make_float4(fmaf(f.x, u.x, -__fmul_rn(f.y, u.y)), fmaf(f.y, u.x, __fmul_rn(f.x, u.y)),
+                                         fmaf(f.x, u.z, -__fmul_rn(f.y, u.w)), fmaf(f.y, u.z, __fmul_rn(f.x, u.w)));
                 }
             }
             __syncthreads();
@@ -456,8 +457,8 @@ __global__ void __launch_bounds__(256, MINB) k_down_win_pp(DevLevel<float> P, De
 // * gam(theta), and gam commutes with the phi interpolation, so the first
 // child's T is scaled by its gam, the second's is scaled and added, and the
 // phi step of the sum is accumulated with the pair's common shift_xy.
-template <int NB, int MINB, bool PAIR = false>
-__global__ void __launch_bounds__(256, MINB) k_up_win(DevLevel<float> P, DevLevel<float> Ch, int B, int RS, int Bs,
+template <int NB, int MINB, bool PAIR = false, int NT = 256>
+__global__ void __launch_bounds__(NT, MINB) k_up_win(DevLevel<float> P, DevLevel<float> Ch, int B, int RS, int Bs,
                                                       int accumulate)
 {
     constexpr int NCP = NB / 2, RL = 32 / NCP, ES = NB / 2;
@@ -543,8 +544,8 @@ __global__ void __launch_bounds__(256, MINB) k_up_win(DevLevel<float> P, DevLeve
                             float4 *t4 = T4 + ((size_t)tt * tpit + v) * NCP + cpi;
                             if (PAIR && rc) {   // scale by the z factor of this child's shift; the second adds
                                 const float2 gz = gam[(int64_t)Ch.octant[c] * ntp + tt];
-                                val = make_float4(gz.x * val.x - gz.y * val.y, gz.x * val.y + gz.y * val.x,
-                                                  gz.x * val.z - gz.y * val.w, gz.x * val.w + gz.y * val.z);
+                                val = make_float4(fmaf(gz.x, val.x, -__fmul_rn(gz.y, val.y)), fmaf(gz.x, val.y, __fmul_rn(gz.y, val.x)),
+                                                  fmaf(gz.x, val.z, -__fmul_rn(gz.y, val.w)), fmaf(gz.x, val.w, __fmul_rn(gz.y, val.z)));
                                 if (rc == 2) {
                                     const float4 old = *t4;
                                     val.x += old.x; val.y += old.y; val.z += old.z; val.w += old.w;
@@ -617,6 +618,7 @@ __global__ void __launch_bounds__(256, MINB) k_up_win(DevLevel<float> P, DevLeve
 }
 
 constexpr size_t kWinSmemCap = 200 * 1024;
+constexpr size_t kUpCap3 = 72 * 1024, kUpCap2 = 100 * 1024;   // up pass: shared memory for three, for two CTAs per SM
 
 size_t down_win_smem(const DevLevel<float> &P, const DevLevel<float> &Ch, int NB)
 {
@@ -634,14 +636,14 @@ size_t up_win_smem(const DevLevel<float> &P, const DevLevel<float> &Ch, int NB, 
 }
 
 // MINB: CTAs per SM the register budget is set for (3 or 4 for down, 2 or 3 for up)
-template <int NB, int MINB, bool PAIR = false>
+template <int NB, int MINB, bool PAIR = false, int NT = 256>
 cudaError_t down_win_nb(const DevLevel<float> &P, const DevLevel<float> &Ch, int B, int Bs, cudaStream_t s)
 {
     const size_t smem = down_win_smem(P, Ch, NB);
     if (smem > kWinSmemCap) return cudaErrorInvalidConfiguration;
     if (PAIR && (!P.dgrp || !P.shift_xy || !P.gam)) return cudaErrorInvalidConfiguration;
     dim3 grid((PAIR ? P.ndgrp : Ch.nbox) * ((B + NB - 1) / NB), 2);
-    k_down_win<NB, MINB, PAIR><<<grid, 256, smem, s>>>(P, Ch, B, Bs);
+    k_down_win<NB, MINB, PAIR, NT><<<grid, NT, smem, s>>>(P, Ch, B, Bs);
     return cudaGetLastError();
 }
 
@@ -661,13 +663,13 @@ cudaError_t down_win_pp_nb(const DevLevel<float> &P, const DevLevel<float> &Ch, 
     return cudaGetLastError();
 }
 
-template <int NB, int MINB, bool PAIR = false>
+template <int NB, int MINB, bool PAIR = false, int NT = 256>
 cudaError_t up_win_nb(const DevLevel<float> &P, const DevLevel<float> &Ch, int B, int Bs, int acc, cudaStream_t s)
 {
     if (PAIR && (!P.shift_xy || !P.gam)) return cudaErrorInvalidConfiguration;
     // bands of parent theta groups: shared memory for MINB CTAs per SM, and
     // enough CTAs to fill the GPU
-    const size_t cap = (size_t)(MINB >= 3 ? 72 : 100) * 1024;
+    const size_t cap = MINB >= 3 ? kUpCap3 : kUpCap2;
     int RS = 1;
     while (RS < P.wu_th.groups && up_win_smem(P, Ch, NB, RS) > cap) ++RS;
     const int64_t ctas = (int64_t)P.nbox * 2 * ((B + NB - 1) / NB);
@@ -675,11 +677,56 @@ cudaError_t up_win_nb(const DevLevel<float> &P, const DevLevel<float> &Ch, int B
     const size_t smem = up_win_smem(P, Ch, NB, RS);
     if (smem > kWinSmemCap) return cudaErrorInvalidConfiguration;
     dim3 grid(P.nbox * ((B + NB - 1) / NB) * RS, 2);
-    k_up_win<NB, MINB, PAIR><<<grid, 256, smem, s>>>(P, Ch, B, RS, Bs, acc);
+    k_up_win<NB, MINB, PAIR, NT><<<grid, NT, smem, s>>>(P, Ch, B, RS, Bs, acc);
     return cudaGetLastError();
 }
 
 bool win_ok(const WinDev &a, const WinDev &b) { return a.groups > 0 && b.groups > 0 && a.coef && b.coef; }
+
+}  // namespace
+
+namespace {
+
+// Columns per CTA of the built-in choice: 8, or 4 where 8 would leave a
+// sixth of the chunks' columns empty.
+bool narrow_chunks(int B) { return 6 * ((B + 3) / 4 * 4) <= 5 * ((B + 7) / 8 * 8); }
+
+constexpr size_t kThird = 74 * 1024;   // down pass: shared memory for three CTAs per SM
+
+// The built-in shapes.  These kernels are bound by the latency of each CTA's
+// chain of phases (issue slots 50-60 % active), so what counts is warps per
+// SM: three CTAs where their fields fit, with 8 columns each if those do
+// (one broadcast coefficient serves more columns), else with 4; a CTA that
+// has the SM to itself or shares it with one other takes 512 threads in the
+// down pass.  Measured (64 columns, us; cube of 8 wavelengths, 6 levels, d0 =
+// 5): down from level 3 (24 x 48 samples) 8 columns, one CTA per SM 1,654,
+// 4 columns, three 1,059; down from level 2 (38 x 76) 4 columns, 256 threads
+// 1,015, 512 threads 847; up into level 2 8 columns 829, 4 columns 724.  Up
+// pass with registers for three CTAs (cube of 4 wavelengths, 14 x 28 samples,
+// 59 KB) 399 against 351, but where only two fit (84 KB) splitting the parent
+// into bands to make room for the third costs more than it gives (1,721
+// against 1,857).
+template <bool PAIR>
+cudaError_t down_win_auto(const DevLevel<float> &P, const DevLevel<float> &Ch, int B, int Bs, cudaStream_t s)
+{
+    if (!narrow_chunks(B) && down_win_smem(P, Ch, 8) <= kThird) return down_win_nb<8, 3, PAIR>(P, Ch, B, Bs, s);
+    if (down_win_smem(P, Ch, 4) <= kThird) return down_win_nb<4, 3, PAIR>(P, Ch, B, Bs, s);
+    return down_win_nb<4, 2, PAIR, 512>(P, Ch, B, Bs, s);
+}
+
+template <bool PAIR>
+cudaError_t up_win_auto(const DevLevel<float> &P, const DevLevel<float> &Ch, int B, int Bs, int acc, cudaStream_t s)
+{
+    if (!narrow_chunks(B)) {
+        const size_t whole = up_win_smem(P, Ch, 8, 1);
+        if (whole <= kUpCap3) return up_win_nb<8, 3, PAIR>(P, Ch, B, Bs, acc, s);
+        if (whole <= kUpCap2) return up_win_nb<8, 2, PAIR>(P, Ch, B, Bs, acc, s);
+        // too few parents to fill the GPU: bands cost nothing, and fewer, wider chunks load the children less often
+        if ((int64_t)P.nbox * 2 * ((B + 7) / 8) <= 2 * 152) return up_win_nb<8, 2, PAIR>(P, Ch, B, Bs, acc, s);
+    }
+    if (up_win_smem(P, Ch, 4, 1) <= kUpCap3) return up_win_nb<4, 3, PAIR>(P, Ch, B, Bs, acc, s);
+    return up_win_nb<4, 2, PAIR>(P, Ch, B, Bs, acc, s);
+}
 
 }  // namespace
 
@@ -688,6 +735,7 @@ cudaError_t launch_down_win(const DevLevel<float> &P, const DevLevel<float> &Ch,
 {
     if (!win_ok(P.wd_ph, P.wd_th) || B < 1) return cudaErrorInvalidConfiguration;
     switch (nb) {
+    case 0: return P.dgrp && P.shift_xy && P.gam ? down_win_auto<true>(P, Ch, B, Bs, s) : down_win_auto<false>(P, Ch, B, Bs, s);
     case 4: return down_win_nb<4, 3>(P, Ch, B, Bs, s);
     case 8: return down_win_nb<8, 3>(P, Ch, B, Bs, s);
     case 16: return down_win_nb<16, 3>(P, Ch, B, Bs, s);
@@ -695,6 +743,7 @@ cudaError_t launch_down_win(const DevLevel<float> &P, const DevLevel<float> &Ch,
     case 108: return down_win_nb<8, 4>(P, Ch, B, Bs, s);
     case 504: return down_win_nb<4, 3, true>(P, Ch, B, Bs, s);
     case 508: return down_win_nb<8, 3, true>(P, Ch, B, Bs, s);
+    case 554: return down_win_nb<4, 2, true, 512>(P, Ch, B, Bs, s);
     case 204: return down_win_pp_nb<4, 3>(P, Ch, B, Bs, s);
     case 208: return down_win_pp_nb<8, 2>(P, Ch, B, Bs, s);
     default: return cudaErrorInvalidConfiguration;
@@ -706,6 +755,7 @@ cudaError_t launch_up_win(const DevLevel<float> &P, const DevLevel<float> &Ch, i
 {
     if (!win_ok(P.wu_th, P.wu_ph) || B < 1) return cudaErrorInvalidConfiguration;
     switch (nb) {
+    case 0: return P.shift_xy && P.gam ? up_win_auto<true>(P, Ch, B, Bs, acc, s) : up_win_auto<false>(P, Ch, B, Bs, acc, s);
     case 4: return up_win_nb<4, 2>(P, Ch, B, Bs, acc, s);
     case 8: return up_win_nb<8, 2>(P, Ch, B, Bs, acc, s);
     case 16: return up_win_nb<16, 2>(P, Ch, B, Bs, acc, s);
@@ -714,6 +764,8 @@ cudaError_t launch_up_win(const DevLevel<float> &P, const DevLevel<float> &Ch, i
     case 404: return up_win_nb<4, 2, true>(P, Ch, B, Bs, acc, s);
     case 408: return up_win_nb<8, 2, true>(P, Ch, B, Bs, acc, s);
     case 416: return up_win_nb<16, 2, true>(P, Ch, B, Bs, acc, s);
+    case 454: return up_win_nb<4, 3, true>(P, Ch, B, Bs, acc, s);
+    case 458: return up_win_nb<8, 3, true>(P, Ch, B, Bs, acc, s);
     default: return cudaErrorInvalidConfiguration;
     }
 }
@@ -725,6 +777,8 @@ cudaError_t prime_win_kernels()
     ALLOW((k_down_win<4, 3>)); ALLOW((k_down_win<8, 3>)); ALLOW((k_down_win<16, 3>));
     ALLOW((k_down_win<4, 4>)); ALLOW((k_down_win<8, 4>));
     ALLOW((k_down_win_pp<4, 3>)); ALLOW((k_down_win_pp<8, 2>));
+    ALLOW((k_down_win<4, 2, false, 512>)); ALLOW((k_down_win<4, 2, true, 512>));
+    ALLOW((k_up_win<4, 3, true>)); ALLOW((k_up_win<8, 3, true>));
     ALLOW((k_down_win<4, 3, true>)); ALLOW((k_down_win<8, 3, true>));
     ALLOW((k_up_win<4, 2>)); ALLOW((k_up_win<8, 2>)); ALLOW((k_up_win<16, 2>));
     ALLOW((k_up_win<4, 3>)); ALLOW((k_up_win<8, 3>));

@@ -1,6 +1,7 @@
 """Built-in kernels that follow the number of columns: register-tiled near
-field, radiation and reception, and the translation.  Column counts at the
-edges of their tiles (1, 2, 4, 16, 32, 64 columns, one less and one more), boxes from one unknown to several
+field, radiation and reception, the flattened translation, and the windowed
+passes' choice of shape.  Column counts at the edges of their tiles (1, 2, 4,
+16, 32, 64 columns, one less and one more), boxes from one unknown to several
 row passes, trees with few leaf boxes (row and sample splits) and many.
 
 Tolerances (relative 2-norms, fixed from the arithmetic): FP32 sums of at most
@@ -80,4 +81,24 @@ def test_columns_agree_with_single_fp64_columns(mesh, levels):
             for c in cols:
                 if c < B:
                     assert rel(y[:, c], one[c]) < 1e-10, (B, c)
+    P.close()
+
+
+def test_builtin_window_shapes_agree_with_pinned_ones():
+    """The built-in up and down shapes against pinned windowed shapes and the
+    new ones (754, 758, 854), for column counts on both sides of the rule:
+    FP32 rounding only."""
+    W = workloads.get("sphere-r2m-ico5")
+    v, t = W.mesh()
+    P = M.MlfmaPlan(v, t, W.k, W.levels, W.digits, max_batch=40, precisions=(M.FP32,))
+    L = M.MAX_LEVELS
+    for B in (2, 3, 9, 12, 13, 16, 36, 40):
+        x = gpu(workloads.rhs(P.n, B, B), torch.float32)
+        P.tune_set(B, np.zeros(M.TUNE_FIELDS, np.int32))
+        y0 = P.matvec(x).cpu().numpy()
+        for u, d in ((304, 304), (754, 854), (758, 804)):
+            c = np.zeros(M.TUNE_FIELDS, np.int32)
+            c[3 + 2], c[3 + 3], c[3 + L + 2], c[3 + L + 3] = u, u, d, d
+            P.tune_set(B, c)
+            assert rel(P.matvec(x).cpu().numpy(), y0) < 1e-5, (B, u, d)
     P.close()
