@@ -1630,7 +1630,7 @@ cudaError_t launch_up(const DevLevel<R> &P, const DevLevel<R> &Ch, int B, int Bs
         else return cudaErrorInvalidConfiguration;
     }
     if constexpr (sizeof(R) == 4) {
-        if (nb_choice == 0 && B >= 2) {   // built-in: windowed, with z pairs where the level has the split shift
+        if (nb_choice == 0 && B >= 1) {   // built-in: windowed, with z pairs where the level has the split shift
             const cudaError_t e = launch_up_win(P, Ch, B, Bs, acc, 0, s);
             if (e != cudaErrorInvalidConfiguration) return e;
         }
@@ -1785,7 +1785,7 @@ cudaError_t launch_down(const DevLevel<R> &P, const DevLevel<R> &Ch, int B, int 
         else return cudaErrorInvalidConfiguration;
     }
     if constexpr (sizeof(R) == 4) {
-        if (nb_choice == 0 && B >= 3) {   // built-in: windowed, with z pairs where the level has the split shift
+        if (nb_choice == 0 && B >= 1) {   // built-in: windowed, with z pairs where the level has the split shift
             const cudaError_t e = launch_down_win(P, Ch, B, Bs, 0, s);
             if (e != cudaErrorInvalidConfiguration) return e;
         }

@@ -18,7 +18,7 @@
 // of 32 columns had cost (30,720-unknown sphere, leaf level) 384 us at 40
 // columns against 240, and (122,880 unknowns) 1,440 us at 34 against 942.
 // Where every quad is whole and aligned, five CTAs without prefetch measured
-// faster (64 columns, 115,200-unknown cube: 1,936 against 1,970 us with the
+// faster (64 columns, 115,200-unknown cube: 1,889 against 1,942 us with the
 // next entry's sources requested ahead in four CTAs); where columns are
 // missing, the loads are longer and requesting ahead wins (34 columns: 942
 // against 1,020).  Tried and slower: packed fma.rn.f32x2 (1,960 to 2,400 us,
@@ -38,40 +38,36 @@ constexpr int kMaxEntries = 216;   // entries of one parent (the plan's bound)
 constexpr int kCh = 4;             // children per pass
 constexpr unsigned kNone = 0xffffu;   // (entry, child) slot without a translation
 
-// Four columns of one field row: two 16-byte loads when all four exist and
-// are aligned, else the existing ones (zero past the end).
-__device__ __forceinline__ void ld_quad(const float2 *p, int cols, bool a16, float4 &lo, float4 &hi)
+// A thread's four columns are two pairs: where every quad is whole, pairs qd
+// and qd + nqd of the row, so that neighbouring threads read neighbouring 16
+// bytes (as four adjacent columns, each 16-byte load of a warp touched twice
+// the lines: 1,936 against 1,889 us, 64 columns of the 115,200-unknown cube);
+// else adjacent ones.
+// One pair of a field row: one 16-byte load when both columns exist and are
+// aligned, else the existing ones (zero past the end).
+__device__ __forceinline__ float4 ld_pair(const float2 *p, int cols, bool a16)
 {
-    if (cols == 4 && a16) {
-        lo = reinterpret_cast<const float4 *>(p)[0];
-        hi = reinterpret_cast<const float4 *>(p)[1];
-        return;
-    }
-    float2 v[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = k < cols ? p[k] : make_float2(0.f, 0.f);
-    lo = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
-    hi = make_float4(v[2].x, v[2].y, v[3].x, v[3].y);
+    if (cols == 2 && a16) return *reinterpret_cast<const float4 *>(p);
+    const float2 u = cols > 0 ? p[0] : make_float2(0.f, 0.f), v = cols > 1 ? p[1] : make_float2(0.f, 0.f);
+    return make_float4(u.x, u.y, v.x, v.y);
 }
 
-__device__ __forceinline__ void st_quad(float2 *p, int cols, bool a16, float4 lo, float4 hi, int accumulate)
+__device__ __forceinline__ void st_pair(float2 *p, int cols, bool a16, float4 v, int accumulate)
 {
-    if (cols == 4 && a16) {
+    if (cols == 2 && a16) {
         float4 *q = reinterpret_cast<float4 *>(p);
         if (accumulate) {
-            const float4 a = q[0], b = q[1];
-            lo.x += a.x; lo.y += a.y; lo.z += a.z; lo.w += a.w;
-            hi.x += b.x; hi.y += b.y; hi.z += b.z; hi.w += b.w;
+            const float4 o = *q;
+            v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
         }
-        q[0] = lo;
-        q[1] = hi;
+        *q = v;
         return;
     }
-    const float2 v[4] = {make_float2(lo.x, lo.y), make_float2(lo.z, lo.w), make_float2(hi.x, hi.y), make_float2(hi.z, hi.w)};
+    const float2 w[2] = {make_float2(v.x, v.y), make_float2(v.z, v.w)};
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
+    for (int k = 0; k < 2; ++k)
         if (k < cols) {
-            float2 y = v[k];
+            float2 y = w[k];
             if (accumulate) {
                 const float2 o = p[k];
                 y.x += o.x;
@@ -122,20 +118,22 @@ __global__ void __launch_bounds__(kThreads, MINB) k_translate_q4(DevLevel<float>
     __syncthreads();
     const int q = (i0 + threadIdx.x) / nqd, qd = i0 + threadIdx.x - q * nqd;
     if (q >= K) return;
-    const int cols = FULL ? 4 : min(4, B - 4 * qd);
-    const float2 *S = reinterpret_cast<const float2 *>(lv.S) + (int64_t)q * Bs + 4 * qd;
+    const int b = FULL ? 2 * qd : 4 * qd, hi = FULL ? 2 * nqd : 2;   // the first pair, and from it to the second
+    const int cl = FULL ? 2 : min(2, B - b), ch = FULL ? 2 : max(0, min(2, B - b - hi));   // their columns
+    const float2 *S = reinterpret_cast<const float2 *>(lv.S) + (int64_t)q * Bs + b;
     const float2 *alq = s_al + (q - q0);
     auto load = [&](int e, float4 (&s)[2][2]) {
         const float2 *src = S + s_off[e];
         if (FULL) {
-            const float4 *p4 = reinterpret_cast<const float4 *>(src), *q4 = reinterpret_cast<const float4 *>(src + KB);
-            s[0][0] = p4[0];
-            s[0][1] = p4[1];
-            s[1][0] = q4[0];
-            s[1][1] = q4[1];
+            s[0][0] = *reinterpret_cast<const float4 *>(src);
+            s[0][1] = *reinterpret_cast<const float4 *>(src + hi);
+            s[1][0] = *reinterpret_cast<const float4 *>(src + KB);
+            s[1][1] = *reinterpret_cast<const float4 *>(src + KB + hi);
         } else {
-            ld_quad(src, cols, a16, s[0][0], s[0][1]);
-            ld_quad(src + KB, cols, a16, s[1][0], s[1][1]);
+            s[0][0] = ld_pair(src, cl, a16);
+            s[0][1] = ld_pair(src + hi, ch, a16);
+            s[1][0] = ld_pair(src + KB, cl, a16);
+            s[1][1] = ld_pair(src + KB + hi, ch, a16);
         }
     };
     for (int c0 = 0; c0 < nc; c0 += kCh) {
@@ -174,13 +172,16 @@ __global__ void __launch_bounds__(kThreads, MINB) k_translate_q4(DevLevel<float>
                 }
             }
         }
-        float2 *G = reinterpret_cast<float2 *>(lv.G) + (int64_t)q * Bs + 4 * qd;
+        float2 *G = reinterpret_cast<float2 *>(lv.G) + (int64_t)q * Bs + b;
 #pragma unroll
         for (int c = 0; c < kCh; ++c) {
             if (c >= nch) break;
 #pragma unroll
-            for (int m = 0; m < 2; ++m)
-                st_quad(G + ((int64_t)(m0 + c0 + c) * 2 + m) * KB, cols, a16, acc[c][m][0], acc[c][m][1], accumulate);
+            for (int m = 0; m < 2; ++m) {
+                float2 *o = G + ((int64_t)(m0 + c0 + c) * 2 + m) * KB;
+                st_pair(o, cl, a16, acc[c][m][0], accumulate);
+                st_pair(o + hi, ch, a16, acc[c][m][1], accumulate);
+            }
         }
     }
 }

@@ -705,10 +705,13 @@ constexpr size_t kThird = 74 * 1024;   // down pass: shared memory for three CTA
 // pass with registers for three CTAs (cube of 4 wavelengths, 14 x 28 samples,
 // 59 KB) 399 against 351, but where only two fit (84 KB) splitting the parent
 // into bands to make room for the third costs more than it gives (1,721
-// against 1,857).
+// against 1,857).  One or two columns take 2 per CTA (30,720-unknown sphere,
+// 2 columns: down from level 3 39 -> 35 us, up 53 -> 51 with 4 per CTA before;
+// 1 column, against the kernel of one row per thread: up 63 -> 51).
 template <bool PAIR>
 cudaError_t down_win_auto(const DevLevel<float> &P, const DevLevel<float> &Ch, int B, int Bs, cudaStream_t s)
 {
+    if (B <= 2 && down_win_smem(P, Ch, 2) <= kThird) return down_win_nb<2, 3, PAIR>(P, Ch, B, Bs, s);
     if (!narrow_chunks(B) && down_win_smem(P, Ch, 8) <= kThird) return down_win_nb<8, 3, PAIR>(P, Ch, B, Bs, s);
     if (down_win_smem(P, Ch, 4) <= kThird) return down_win_nb<4, 3, PAIR>(P, Ch, B, Bs, s);
     return down_win_nb<4, 2, PAIR, 512>(P, Ch, B, Bs, s);
@@ -717,6 +720,7 @@ cudaError_t down_win_auto(const DevLevel<float> &P, const DevLevel<float> &Ch, i
 template <bool PAIR>
 cudaError_t up_win_auto(const DevLevel<float> &P, const DevLevel<float> &Ch, int B, int Bs, int acc, cudaStream_t s)
 {
+    if (B <= 2 && up_win_smem(P, Ch, 2, 1) <= kUpCap3) return up_win_nb<2, 3, PAIR>(P, Ch, B, Bs, acc, s);
     if (!narrow_chunks(B)) {
         const size_t whole = up_win_smem(P, Ch, 8, 1);
         if (whole <= kUpCap3) return up_win_nb<8, 3, PAIR>(P, Ch, B, Bs, acc, s);
@@ -777,6 +781,7 @@ cudaError_t prime_win_kernels()
     ALLOW((k_down_win<4, 3>)); ALLOW((k_down_win<8, 3>)); ALLOW((k_down_win<16, 3>));
     ALLOW((k_down_win<4, 4>)); ALLOW((k_down_win<8, 4>));
     ALLOW((k_down_win_pp<4, 3>)); ALLOW((k_down_win_pp<8, 2>));
+    ALLOW((k_down_win<2, 3, false>)); ALLOW((k_down_win<2, 3, true>)); ALLOW((k_up_win<2, 3, false>)); ALLOW((k_up_win<2, 3, true>));
     ALLOW((k_down_win<4, 2, false, 512>)); ALLOW((k_down_win<4, 2, true, 512>));
     ALLOW((k_up_win<4, 3, true>)); ALLOW((k_up_win<8, 3, true>));
     ALLOW((k_down_win<4, 3, true>)); ALLOW((k_down_win<8, 3, true>));

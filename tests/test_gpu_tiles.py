@@ -92,7 +92,7 @@ def test_builtin_window_shapes_agree_with_pinned_ones():
     v, t = W.mesh()
     P = M.MlfmaPlan(v, t, W.k, W.levels, W.digits, max_batch=40, precisions=(M.FP32,))
     L = M.MAX_LEVELS
-    for B in (2, 3, 9, 12, 13, 16, 36, 40):
+    for B in (1, 2, 3, 9, 12, 13, 16, 36, 40):
         x = gpu(workloads.rhs(P.n, B, B), torch.float32)
         P.tune_set(B, np.zeros(M.TUNE_FIELDS, np.int32))
         y0 = P.matvec(x).cpu().numpy()
