@@ -938,7 +938,7 @@ mlfma_status core_graph(mlfma_plan_t p, const ProductArgs<R> &a, int prec, int k
     }
     cudaError_t e = cudaStreamBeginCapture(p->cs.main, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(e, "graph capture");
-    cudaError_t el = dk ? launch_core_dk<R>(a, p->cs.main, nullptr) : launch_core<R>(a, p->cs, nullptr);
+    cudaError_t el = dk ? launch_core_dk<R>(a, p->cs, nullptr) : launch_core<R>(a, p->cs, nullptr);
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(p->cs.main, &g);
     if (el != cudaSuccess || e != cudaSuccess) {
@@ -977,7 +977,7 @@ mlfma_status run(mlfma_plan_t p, ProductArgs<R> a, int prec, const void *xd, int
         if ((e = launch_prepare<R>(a, xd, xc, Bu, adjoint, s)) != cudaSuccess) return cuda_fail(e, "prepare");
         clk.stage[clk.n] = STAGE_PREPARE;
         if ((e = cudaEventRecord(clk.ev[clk.n++], s)) != cudaSuccess) return cuda_fail(e, "stage timer");
-        if ((e = dk ? launch_core_dk<R>(a, s, &clk) : launch_core<R>(a, serial, &clk)) != cudaSuccess)
+        if ((e = dk ? launch_core_dk<R>(a, serial, &clk) : launch_core<R>(a, serial, &clk)) != cudaSuccess)
             return cuda_fail(e, "core pass");
         if ((e = launch_finalize<R>(a, yd, xc, Bu, adjoint, s)) != cudaSuccess) return cuda_fail(e, "finalize");
         clk.stage[clk.n] = STAGE_FINALIZE;

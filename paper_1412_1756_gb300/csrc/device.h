@@ -236,10 +236,9 @@ template <class R>
 cudaError_t launch_core(const ProductArgs<R> &a, const CoreStreams &cs, StageClock *clk);
 // (dZ/dk) x into a.yp: the near blocks of dZ/dk, and the far pass carried as
 // value and k-tangent side by side (fields hold 2 a.B columns: value in
-// [0, a.B), tangent in [a.B, 2 a.B)); on one stream, an event per stage
-// with clk.
+// [0, a.B), tangent in [a.B, 2 a.B)); streams and clk as launch_core.
 template <class R>
-cudaError_t launch_core_dk(const ProductArgs<R> &a, cudaStream_t s, StageClock *clk);
+cudaError_t launch_core_dk(const ProductArgs<R> &a, const CoreStreams &cs, StageClock *clk);
 
 // One stage of the core pass with a given choice (mlfma_tune): stage is
 // STAGE_NEAR, STAGE_RADIATE, STAGE_RECEIVE, STAGE_UP + l, STAGE_TRANSLATE + l

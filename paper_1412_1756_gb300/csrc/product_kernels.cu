@@ -1967,6 +1967,16 @@ cudaError_t launch_core_streams(const ProductArgs<R> &a, const CoreStreams &cs, 
     return cudaSuccess;
 }
 
+namespace {
+void join_side_streams(const CoreStreams &cs)
+{
+    const cudaStream_t side[2] = {cs.far, cs.tr};
+    for (int i = 0; i < 2; ++i)
+        if (side[i] && cudaEventRecord(cs.ev[62 + i], side[i]) == cudaSuccess)
+            cudaStreamWaitEvent(cs.main, cs.ev[62 + i], 0);
+}
+}  // namespace
+
 // The concurrent pass above; when a launch fails part way, the side streams
 // are joined back into the main one (so that a stream capture in progress
 // can end, and no stream is left forked) and the failure is returned.
@@ -1974,12 +1984,7 @@ template <class R>
 cudaError_t launch_core(const ProductArgs<R> &a, const CoreStreams &cs, StageClock *clk)
 {
     const cudaError_t e = launch_core_streams<R>(a, cs, clk);
-    if (e != cudaSuccess && clk == nullptr && cs.far != nullptr) {
-        const cudaStream_t side[2] = {cs.far, cs.tr};
-        for (int i = 0; i < 2; ++i)
-            if (side[i] && cudaEventRecord(cs.ev[62 + i], side[i]) == cudaSuccess)
-                cudaStreamWaitEvent(cs.main, cs.ev[62 + i], 0);
-    }
+    if (e != cudaSuccess && clk == nullptr && cs.far != nullptr) join_side_streams(cs);
     return e;
 }
 
@@ -1994,71 +1999,106 @@ cudaError_t launch_core(const ProductArgs<R> &a, const CoreStreams &cs, StageClo
 //   down       G_c' += Anterp(conj(shift'_pc) G_p)
 //   receive    y += w conj(V) . G' + w conj(V' + (2/k) V) . G
 // (the 2/k is the derivative of the far constant -k^2 eta / 4 pi over itself).
+//
+// Branches as in launch_core_streams: the near blocks beside the far chain,
+// and each level's two translations as soon as both halves of its outgoing
+// field exist (the tangent's adds to the value's, so they stay in order on
+// one stream).  In one stream, small products left most SMs idle (10,680
+// unknowns, 8 columns: 494 us, in branches 457).
 template <class R>
-cudaError_t launch_core_dk(const ProductArgs<R> &a, cudaStream_t s, StageClock *clk)
+cudaError_t launch_core_dk_streams(const ProductArgs<R> &a, const CoreStreams &cs, StageClock *clk)
 {
     const int T = a.B, Bs = 2 * a.B, leaf = a.leaf;
     if (!a.near_dk || (leaf >= 2 && (!a.Vd || !a.Wd))) return cudaErrorInvalidValue;
+    const bool serial = clk != nullptr || cs.far == nullptr;
+    cudaStream_t s0 = cs.main, sf = serial ? s0 : cs.far, st = serial ? s0 : cs.tr;
     auto tangent = [&](R *f) { return f + 2 * (size_t)T; };   // T complex columns
     cudaError_t e;
 #define TRY(x) do { if ((e = (x)) != cudaSuccess) return e; } while (0)
+    // events: 0 fork, 1 far done, 2 translations done, 3 + l outgoing field of level l ready
+    if (!serial) {
+        TRY(cudaEventRecord(cs.ev[0], s0));
+        TRY(cudaStreamWaitEvent(sf, cs.ev[0], 0));
+    }
     {
         ProductArgs<R> an = a;
         an.near_val = a.near_dk;
-        TRY(launch_near<R>(an, s));
-        TRY(tick(clk, STAGE_NEAR, s));
+        TRY(launch_near<R>(an, s0));
+        TRY(tick(clk, STAGE_NEAR, s0));
     }
-    if (leaf < 2) return cudaSuccess;
-    {
-        TRY(launch_radiate<R>(a, Bs, s));
-        ProductArgs<R> ad = a;
-        ad.V = a.Vd;
-        ad.lv[leaf].S = tangent(a.lv[leaf].S);
-        TRY(launch_radiate<R>(ad, Bs, s));
-        TRY(tick(clk, STAGE_RADIATE, s));
+    if (leaf >= 2) {
+        {
+            TRY(launch_radiate<R>(a, Bs, sf));
+            ProductArgs<R> ad = a;
+            ad.V = a.Vd;
+            ad.lv[leaf].S = tangent(a.lv[leaf].S);
+            TRY(launch_radiate<R>(ad, Bs, sf));
+            TRY(tick(clk, STAGE_RADIATE, sf));
+        }
+        auto translate = [&](int l) -> cudaError_t {
+            cudaError_t e2;
+            if (!serial) {
+                if ((e2 = cudaEventRecord(cs.ev[3 + l], sf)) != cudaSuccess) return e2;
+                if ((e2 = cudaStreamWaitEvent(st, cs.ev[3 + l], 0)) != cudaSuccess) return e2;
+            }
+            if ((e2 = launch_translate<R>(a.lv[l], Bs, Bs, 0, st)) != cudaSuccess) return e2;
+            DevLevel<R> x = a.lv[l];
+            x.alpha = a.lv[l].alpha_dk;
+            x.G = tangent(a.lv[l].G);
+            if ((e2 = launch_translate<R>(x, T, Bs, 1, st)) != cudaSuccess) return e2;
+            return tick(clk, STAGE_TRANSLATE + l, st);
+        };
+        TRY(translate(leaf));
+        for (int l = leaf - 1; l >= 2; --l) {
+            TRY(launch_up<R>(a.lv[l], a.lv[l + 1], Bs, Bs, 0, sf));
+            DevLevel<R> px = a.lv[l];
+            px.shift = a.lv[l].shift_dk;
+            px.shift_xy = px.gam = nullptr;   // the split shift is the value's: no pair kernels here
+            px.dgrp = nullptr;
+            px.S = tangent(a.lv[l].S);
+            TRY(launch_up<R>(px, a.lv[l + 1], T, Bs, 1, sf));
+            TRY(tick(clk, STAGE_UP + l, sf));
+            TRY(translate(l));
+        }
+        if (!serial) {
+            TRY(cudaEventRecord(cs.ev[2], st));
+            TRY(cudaStreamWaitEvent(sf, cs.ev[2], 0));
+        }
+        for (int l = 2; l < leaf; ++l) {
+            TRY(launch_down<R>(a.lv[l], a.lv[l + 1], Bs, Bs, sf));
+            DevLevel<R> px = a.lv[l], cx = a.lv[l + 1];
+            px.shift = a.lv[l].shift_dk;
+            px.shift_xy = px.gam = nullptr;   // the split shift is the value's: no pair kernels here
+            px.dgrp = nullptr;
+            cx.G = tangent(a.lv[l + 1].G);
+            TRY(launch_down<R>(px, cx, T, Bs, sf));
+            TRY(tick(clk, STAGE_DOWN + l, sf));
+        }
     }
-    auto translate = [&](int l) -> cudaError_t {
-        cudaError_t e2 = launch_translate<R>(a.lv[l], Bs, Bs, 0, s);
-        if (e2 != cudaSuccess) return e2;
-        DevLevel<R> x = a.lv[l];
-        x.alpha = a.lv[l].alpha_dk;
-        x.G = tangent(a.lv[l].G);
-        if ((e2 = launch_translate<R>(x, T, Bs, 1, s)) != cudaSuccess) return e2;
-        return tick(clk, STAGE_TRANSLATE + l, s);
-    };
-    TRY(translate(leaf));
-    for (int l = leaf - 1; l >= 2; --l) {
-        TRY(launch_up<R>(a.lv[l], a.lv[l + 1], Bs, Bs, 0, s));
-        DevLevel<R> px = a.lv[l];
-        px.shift = a.lv[l].shift_dk;
-        px.shift_xy = px.gam = nullptr;   // the split shift is the value's: no pair kernels here
-        px.dgrp = nullptr;
-        px.S = tangent(a.lv[l].S);
-        TRY(launch_up<R>(px, a.lv[l + 1], T, Bs, 1, s));
-        TRY(tick(clk, STAGE_UP + l, s));
-        TRY(translate(l));
+    if (!serial) {
+        TRY(cudaEventRecord(cs.ev[1], sf));
+        TRY(cudaStreamWaitEvent(s0, cs.ev[1], 0));
     }
-    for (int l = 2; l < leaf; ++l) {
-        TRY(launch_down<R>(a.lv[l], a.lv[l + 1], Bs, Bs, s));
-        DevLevel<R> px = a.lv[l], cx = a.lv[l + 1];
-        px.shift = a.lv[l].shift_dk;
-        px.shift_xy = px.gam = nullptr;   // the split shift is the value's: no pair kernels here
-        px.dgrp = nullptr;
-        cx.G = tangent(a.lv[l + 1].G);
-        TRY(launch_down<R>(px, cx, T, Bs, s));
-        TRY(tick(clk, STAGE_DOWN + l, s));
-    }
-    {
+    if (leaf >= 2) {
         ProductArgs<R> at = a;
         at.lv[leaf].G = tangent(a.lv[leaf].G);
-        TRY(launch_receive<R>(at, Bs, s));
+        TRY(launch_receive<R>(at, Bs, s0));
         ProductArgs<R> aw = a;
         aw.V = a.Wd;
-        TRY(launch_receive<R>(aw, Bs, s));
-        TRY(tick(clk, STAGE_RECEIVE, s));
+        TRY(launch_receive<R>(aw, Bs, s0));
+        TRY(tick(clk, STAGE_RECEIVE, s0));
     }
 #undef TRY
     return cudaSuccess;
+}
+
+// A failure part way joins the side streams back, as in launch_core.
+template <class R>
+cudaError_t launch_core_dk(const ProductArgs<R> &a, const CoreStreams &cs, StageClock *clk)
+{
+    const cudaError_t e = launch_core_dk_streams<R>(a, cs, clk);
+    if (e != cudaSuccess && clk == nullptr && cs.far != nullptr) join_side_streams(cs);
+    return e;
 }
 
 template <class R>
@@ -2094,9 +2134,9 @@ template cudaError_t launch_finalize<float>(const ProductArgs<float> &, void *, 
 template cudaError_t launch_finalize<double>(const ProductArgs<double> &, void *, int, int, int, cudaStream_t);
 template cudaError_t launch_core<float>(const ProductArgs<float> &, const CoreStreams &, StageClock *);
 template cudaError_t launch_core<double>(const ProductArgs<double> &, const CoreStreams &, StageClock *);
-template cudaError_t launch_core_dk<float>(const ProductArgs<float> &, cudaStream_t, StageClock *);
+template cudaError_t launch_core_dk<float>(const ProductArgs<float> &, const CoreStreams &, StageClock *);
 template cudaError_t launch_stage<float>(const ProductArgs<float> &, int, int, cudaStream_t);
 template cudaError_t launch_stage<double>(const ProductArgs<double> &, int, int, cudaStream_t);
-template cudaError_t launch_core_dk<double>(const ProductArgs<double> &, cudaStream_t, StageClock *);
+template cudaError_t launch_core_dk<double>(const ProductArgs<double> &, const CoreStreams &, StageClock *);
 
 }  // namespace mlfma
