@@ -33,8 +33,9 @@
 // -> 59, 40 columns 250 -> 192; 122,880 unknowns, 34 columns 818 -> 537;
 // 115,200-unknown cube, 64 columns 1,307 -> 1,230.  One column (35 against 61
 // on 28,800 unknowns) and exactly 16 (61 against 76 on 10,824) stay with the
-// older kernels.  FP64, 1,920 unknowns, 8 columns 186 -> 80; below three
-// columns the older kernels win (28,800 unknowns, 2 columns 409 against 440).
+// older kernels.  FP64, 1,920 unknowns, 8 columns 186 -> 80; up to four
+// columns k_receive wins unless boxes are few (28,800 unknowns, 2 columns 325
+// against 440).
 #include "device.h"
 
 #include <algorithm>
@@ -408,7 +409,7 @@ cudaError_t receive_go(const ProductArgs<R> &a, int Bs, int ncp, cudaStream_t s)
     const int least = (2 * QT * ncp + NE - 1) / NE;   // NE field elements per thread and tile
     const int threads = split ? 256 : std::min(256, (std::max({64, nct * want, least}) + 31) / 32 * 32);
     const int RP = std::min((a.nr.max_rows + kRows - 1) / kRows, threads / nct) * kRows;
-    if (2 * QT * ncp > NE * threads) return cudaErrorInvalidConfiguration;
+    if (2 * QT * ncp > NE * threads || (int64_t)2 * Lf.K * Bs > INT32_MAX) return cudaErrorInvalidConfiguration;   // 32-bit field offsets
     const size_t stage = (size_t)4 * QT * ncp * sizeof(Cols<R, CW>) + (size_t)2 * RP * (QT + 1) * sizeof(Four<R>);
     const size_t part = split ? (size_t)256 * kRows * CW * 2 * sizeof(R) : 0;
     const size_t smem = std::max(stage, part);

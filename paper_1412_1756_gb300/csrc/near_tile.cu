@@ -209,7 +209,7 @@ cudaError_t go(const ProductArgs<R> &a, int nbc, cudaStream_t s)
     const uintptr_t align = reinterpret_cast<uintptr_t>(a.xp) | ((uintptr_t)a.B * sizeof(R)) | ((uintptr_t)chunk * sizeof(R)) |
                             ((uintptr_t)(a.B % chunk) * sizeof(R)) | ((uintptr_t)XP * sizeof(R));
     const int xu = (align & 15) == 0 ? 16 : (align & 7) == 0 ? 8 : 4;
-    if (xu < (int)sizeof(R)) return cudaErrorInvalidConfiguration;
+    if (xu < (int)sizeof(R) || (reinterpret_cast<uintptr_t>(a.near_val) & 15) != 0) return cudaErrorInvalidConfiguration;
     int lsh = 0;
     while (lsh < 5 && (1 << lsh) < chunk * (int)sizeof(R) / xu) ++lsh;
     const int64_t ctas = (int64_t)a.nr.nleaf * nch;

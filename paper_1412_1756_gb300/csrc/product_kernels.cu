@@ -1079,8 +1079,13 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && TM <= 20) ? 2 : 1)
 // ------------------------------------------------------------ receive ---
 // y_i += sum_q wq_q conj(V_s,mi(q)) . G_m(q).
 // Few columns: one CTA per (leaf box, chunk of LB columns) with the box's G
-// block in shared memory; one warp per unknown at a time, lanes split into
-// LB column lanes x 32/LB sample lanes, reduced with shuffles.
+// block, scaled by the weights, in shared memory; a warp takes two unknowns at
+// a time, lanes split into LB column lanes x 32/LB sample lanes, reduced with
+// shuffles (the first step leaves each half of the lanes one unknown).  FP64
+// is bound by its arithmetic, so what counts is operations: weights per
+// sample and unknown and five shuffle steps per unknown had made 100 of the
+// 72 that one unknown's 288 samples need (28,800 unknowns, 1 column, 224 us;
+// now 162.  2 columns 416 -> 325).
 template <class R, int LB>
 __global__ void __launch_bounds__(256) k_receive(const int32_t *__restrict__ box_ptr,
                                                  const typename Cx<R>::T4 *__restrict__ V4, DevLevel<R> lf,
@@ -1098,35 +1103,58 @@ __global__ void __launch_bounds__(256) k_receive(const int32_t *__restrict__ box
     const int nb = min(LB, B - b0);
     const C *G = reinterpret_cast<const C *>(lf.G) + (int64_t)box * 2 * K * Bs + b0;
     for (int e = threadIdx.x; e < 2 * K * LB; e += blockDim.x) {
-        const int bb = e % LB;
-        Gs[e] = bb < nb ? G[(int64_t)(e / LB) * Bs + bb] : C{0, 0};
+        const int bb = e % LB, mq = e / LB;
+        C g = bb < nb ? G[(int64_t)mq * Bs + bb] : C{0, 0};
+        const R w = lf.wq[mq < K ? mq : mq - K];
+        g.x *= w;
+        g.y *= w;
+        Gs[e] = g;
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     const int lb = lane % LB, lq = lane / LB;
     const int i0 = box_ptr[box], i1 = box_ptr[box + 1];
-    for (int i = i0 + warp; i < i1; i += nwarp) {
+    auto add = [&](int i, C s) {
+        C y = yp[(int64_t)i * B + b0 + lb];
+        y.x += s.x;
+        y.y += s.y;
+        yp[(int64_t)i * B + b0 + lb] = y;
+    };
+    for (int i = i0 + 2 * warp; i < i1; i += 2 * nwarp) {
+        const bool two = i + 1 < i1;
         const C4 *v = V4 + (int64_t)i * K;
-        C acc{0, 0};
+        C a{0, 0}, c{0, 0};
+        if (two) {
 #pragma unroll 4
-        for (int q = lq; q < K; q += LQ) {
-            const C4 vq = v[q];
-            C t{0, 0};
-            cfmac(t, C{vq.x, vq.y}, Gs[q * LB + lb]);
-            cfmac(t, C{vq.z, vq.w}, Gs[(K + q) * LB + lb]);
-            rfma(acc, lf.wq[q], t);
+            for (int q = lq; q < K; q += LQ) {
+                const C4 va = v[q], vc = v[K + q];
+                const C g0 = Gs[q * LB + lb], g1 = Gs[(K + q) * LB + lb];
+                cfmac(a, C{va.x, va.y}, g0);
+                cfmac(c, C{vc.x, vc.y}, g0);
+                cfmac(a, C{va.z, va.w}, g1);
+                cfmac(c, C{vc.z, vc.w}, g1);
+            }
+            const bool upper = lane & 16;   // the upper half of the lanes goes on with the second unknown
+            const R sx = upper ? a.x : c.x, sy = upper ? a.y : c.y;
+            a.x = (upper ? c.x : a.x) + __shfl_xor_sync(0xffffffffu, sx, 16);
+            a.y = (upper ? c.y : a.y) + __shfl_xor_sync(0xffffffffu, sy, 16);
+        } else {
+#pragma unroll 4
+            for (int q = lq; q < K; q += LQ) {
+                const C4 va = v[q];
+                cfmac(a, C{va.x, va.y}, Gs[q * LB + lb]);
+                cfmac(a, C{va.z, va.w}, Gs[(K + q) * LB + lb]);
+            }
+            a.x += __shfl_xor_sync(0xffffffffu, a.x, 16);
+            a.y += __shfl_xor_sync(0xffffffffu, a.y, 16);
         }
 #pragma unroll
-        for (int off = 16; off >= LB; off >>= 1) {
-            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
-            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
+        for (int off = 8; off >= LB; off >>= 1) {
+            a.x += __shfl_xor_sync(0xffffffffu, a.x, off);
+            a.y += __shfl_xor_sync(0xffffffffu, a.y, off);
         }
-        if (lq == 0 && lb < nb) {
-            C y = yp[(int64_t)i * B + b0 + lb];
-            y.x += acc.x;
-            y.y += acc.y;
-            yp[(int64_t)i * B + b0 + lb] = y;
-        }
+        // LB <= 4 column lanes: lanes 0 .. LB - 1 hold the first unknown, lanes 16 .. 16 + LB - 1 the second
+        if (lb < nb && (lane & 15) < LB && (lane < 16 || two)) add(i + (lane >> 4), a);
     }
 }
 
@@ -1538,7 +1566,7 @@ cudaError_t launch_receive(const ProductArgs<R> &a, int Bs, cudaStream_t s, int 
     if (choice == 0) {
         // register tiles that follow the columns (leaf_tile.cu has the figures of both sides); one full chunk of 16
         // is left to the 16-column kernel
-        if (sizeof(R) == 8 ? a.B >= 3 : (a.B >= 2 && a.B != 16)) {
+        if (sizeof(R) == 8 ? (a.B >= 5 || (a.B >= 3 && few_boxes(a.lv[a.leaf].nbox, a.B))) : (a.B >= 2 && a.B != 16)) {
             const cudaError_t e = launch_receive_tile<R>(a, Bs, s);
             if (e != cudaErrorInvalidConfiguration) return e;
         }
