@@ -217,6 +217,15 @@ __device__ __forceinline__ void stage_field(float *raw, const float *src, int K,
     }
 }
 
+// Two warpgroups per CTA: staging the operands and reading the results back
+// bound these kernels (the tensor pipe is active 1-2 % of the time), and
+// where shared memory leaves room for one or two CTAs per SM the copies are
+// shared out over twice the warps - both groups reach the same tensor-memory
+// lanes and split the columns, tiles or K blocks.  3xTF32, one -> two
+// warpgroups (us): 10,680 unknowns, 16 columns, down 236 -> 148 and 252 ->
+// 166, up 90 -> 68 and 100 -> 88; 28,800 unknowns, 64 columns, down from
+// level 2 2,151 -> 1,294.  Up levels whose CTAs fit three to an SM keep one
+// (28,800 unknowns, up into level 3 947 against 1,039).
 // The tensor-memory allocation, operand images and the shared A tile buffer
 // (steps 1 and 2 never hold it at the same time).
 struct Ctx {
@@ -300,17 +309,18 @@ __device__ __forceinline__ void sync_tmem()
 }
 
 // ------------------------------------------------------------------- up ---
-// grid (parent box, component, column-chunk group); 128 threads.  The work
+// grid (parent box, component, column-chunk group); NT threads.  The work
 // items are (chunk, child) pairs; the next item's child field is copied in
 // (cp.async) while the current one is interpolated, and each phi tile's
 // phase shifts while its MMAs run.
-template <bool SPLIT>
-__global__ void __launch_bounds__(128) k_up_umma(DevLevel<float> P, DevLevel<float> Ch, int B, int Bs, int accumulate,
+template <bool SPLIT, int NT>
+__global__ void __launch_bounds__(NT, NT == 128 ? 3 : 2) k_up_umma(DevLevel<float> P, DevLevel<float> Ch, int B, int Bs, int accumulate,
                                                  int cpc)
 {
     extern __shared__ unsigned char smraw[];
     __shared__ uint64_t bar;
     __shared__ uint32_t tslot;
+    constexpr int WG = NT / 128;   // warpgroups
     unsigned char *sm = align1024(smraw);
     const UmmaStep s1 = P.um_up1, s2 = P.um_up2;
     const int tiles1 = (Ch.nth + 15) / 16, tiles2 = (P.nph + 15) / 16;
@@ -322,7 +332,8 @@ __global__ void __launch_bounds__(128) k_up_umma(DevLevel<float> P, DevLevel<flo
     float *const raw0 = reinterpret_cast<float *>(c.rest);   // two buffers of Kc samples x 8 floats
     auto raw = [&](int i) { return raw0 + (size_t)(i & 1) * Kc * 8; };
     float2 *sb = reinterpret_cast<float2 *>(c.rest + (size_t)2 * Kc * 32);   // [N2][16] phase shifts of a phi tile
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = (tid >> 5) & 3, wg = tid >> 7;   // tensor-memory lanes of the warp; warpgroup
     const uint32_t lanes = (uint32_t)(warp * 32) << 16;
     const int p = blockIdx.x, comp = blockIdx.y;
     const int ch0 = P.child_ptr[p], nch = P.child_ptr[p + 1] - ch0;
@@ -353,7 +364,7 @@ __global__ void __launch_bounds__(128) k_up_umma(DevLevel<float> P, DevLevel<flo
         const float *r = raw(it);
         // step 1 (phi), tile by tile of child theta rows
         for (int t1 = 0; t1 < tiles1 && ok; ++t1) {
-            for (int g = warp; g < 16 * (s1.K / 4); g += 4) {
+            for (int g = tid >> 5; g < 16 * (s1.K / 4); g += NT / 32) {
                 const int rg = g & 15, k = (g >> 4) * 4 + klo;
                 const int thc = t1 * 16 + rg;
                 const float v = (thc < nthc && k < nphc) ? r[(thc * nphc + k) * 8 + rsub] : 0.0f;
@@ -375,10 +386,13 @@ __global__ void __launch_bounds__(128) k_up_umma(DevLevel<float> P, DevLevel<flo
             for (int t1 = 0; t1 < tiles1; ++t1) {
                 const int thc = t1 * 16 + warp * 4 + klo;
                 float v[16];
-                tld16(c.tmem + lanes + cD1 + t1 * s1.N + php0, v);
-                if (thc < nthc) {
+                if (WG == 1 || wg == 0) {   // of two warpgroups, the first moves the samples, the second those at phi + pi
+                    tld16(c.tmem + lanes + cD1 + t1 * s1.N + php0, v);
+                    if (thc < nthc) {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) put<SPLIT>(c.ah, c.al, kmaj(i * 8 + rsub, thc, kTile), v[i]);
+                        for (int i = 0; i < 16; ++i) put<SPLIT>(c.ah, c.al, kmaj(i * 8 + rsub, thc, kTile), v[i]);
+                    }
+                    if (WG == 2) continue;
                 }
                 const int kr = s2.kr0 + thc;
                 const bool need = thc < nthc && ((s2.kmask >> (kr >> 3)) & 1u);
@@ -396,7 +410,7 @@ __global__ void __launch_bounds__(128) k_up_umma(DevLevel<float> P, DevLevel<flo
             __syncthreads();
             // shift and accumulate: this thread's row is (php, column, re/im)
             const int pl = warp * 4 + klo;
-            for (int n0 = 0; n0 < s2.N; n0 += 16) {
+            for (int n0 = 16 * wg; n0 < s2.N; n0 += 16 * WG) {
                 float v[16], a[16];
                 tld16(c.tmem + lanes + cD2 + n0, v);
                 if (first) {
@@ -421,7 +435,7 @@ __global__ void __launch_bounds__(128) k_up_umma(DevLevel<float> P, DevLevel<flo
         float *dst = P.S + ((size_t)(p * 2 + comp) * P.K) * Bs * 2;
         for (int t2 = 0; t2 < tiles2; ++t2) {
             const int php = t2 * 16 + warp * 4 + klo;
-            for (int n0 = 0; n0 < s2.N; n0 += 16) {
+            for (int n0 = 16 * wg; n0 < s2.N; n0 += 16 * WG) {
                 float a[16];
                 tld16(c.tmem + lanes + cAcc + t2 * s2.N + n0, a);
                 if (php < nphp && bok) {
@@ -452,14 +466,14 @@ __global__ void __launch_bounds__(128) k_up_umma(DevLevel<float> P, DevLevel<flo
 }
 
 // ----------------------------------------------------------------- down ---
-// grid (child box, component, column-chunk group); 128 threads.  The
+// grid (child box, component, column-chunk group); 256 threads.  The
 // child's phase shifts are copied in once; the parent field of each column
 // chunk is copied in (cp.async) ahead of its use: the next chunk's while this
 // one is worked on (nbuf = 2), or during this one's second step (nbuf = 1).
 // The parent field rows (one theta) are padded by one sample so that a warp
 // reading four theta rows of one phi hits distinct banks.
 template <bool SPLIT>
-__global__ void __launch_bounds__(128) k_down_umma(DevLevel<float> P, DevLevel<float> Ch, int B, int Bs, int cpc,
+__global__ void __launch_bounds__(256, 2) k_down_umma(DevLevel<float> P, DevLevel<float> Ch, int B, int Bs, int cpc,
                                                    int nbuf)
 {
     extern __shared__ unsigned char smraw[];
@@ -477,7 +491,8 @@ __global__ void __launch_bounds__(128) k_down_umma(DevLevel<float> P, DevLevel<f
     float2 *shs = reinterpret_cast<float2 *>(c.rest);      // [Kp] this child's phase shifts
     float *const raw0 = reinterpret_cast<float *>(c.rest + (size_t)Kp * 8);
     auto raw = [&](int i) { return raw0 + (size_t)(i & 1) * nthp * rowp; };
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = (tid >> 5) & 3, wg = tid >> 7;   // tensor-memory lanes of the warp; warpgroup
     const uint32_t lanes = (uint32_t)(warp * 32) << 16;
     const int chd = blockIdx.x, comp = blockIdx.y;
     const int par = Ch.parent[chd], oct = Ch.octant[chd];
@@ -503,7 +518,7 @@ __global__ void __launch_bounds__(128) k_down_umma(DevLevel<float> P, DevLevel<f
         __syncthreads();
         // step 1 (theta), tile by tile of parent phi samples: rows (php, column, re/im)
         for (int t1 = 0; t1 < tiles1 && ok; ++t1) {
-            for (int gi = warp; gi < 16 * (s1.K / 4); gi += 4) {
+            for (int gi = tid >> 5; gi < 16 * (s1.K / 4); gi += 256 / 32) {
                 const int rg = gi & 15, k = (gi >> 4) * 4 + klo;
                 const int php = t1 * 16 + rg;
                 int thp = -1, ph = php;
@@ -528,7 +543,7 @@ __global__ void __launch_bounds__(128) k_down_umma(DevLevel<float> P, DevLevel<f
         }
         // step 2 (phi), tile by tile of child theta rows
         for (int t2 = 0; t2 < tiles2 && ok; ++t2) {
-            for (int t1 = 0; t1 < tiles1; ++t1) {
+            for (int t1 = wg; t1 < tiles1; t1 += 2) {
                 const int php = t1 * 16 + warp * 4 + klo;
                 float v[16];
                 tld16(c.tmem + lanes + cD1 + t1 * s1.N + t2 * 16, v);
@@ -540,7 +555,7 @@ __global__ void __launch_bounds__(128) k_down_umma(DevLevel<float> P, DevLevel<f
             ok = run_step<SPLIT>(c.tmem + cD2, c, true, s2, &bar, phase, false);
             if (!ok) break;
             const int thc = t2 * 16 + warp * 4 + klo;
-            for (int n0 = 0; n0 < s2.N; n0 += 16) {
+            for (int n0 = 16 * wg; n0 < s2.N; n0 += 32) {
                 float v[16];
                 tld16(c.tmem + lanes + cD2 + n0, v);
                 if (thc < nthc && bok) {
@@ -608,15 +623,13 @@ cudaError_t launch_up_umma(const DevLevel<float> &P, const DevLevel<float> &Ch, 
     const int cpc = chunks_per_cta(P.nbox, B);
     const int chunks = (B + kCols - 1) / kCols;
     dim3 grid(P.nbox, 2, (chunks + cpc - 1) / cpc);
-    cudaError_t e;
-    if (split) {
-        if ((e = allow(k_up_umma<true>, smem)) != cudaSuccess) return e;
-        k_up_umma<true><<<grid, 128, smem, s>>>(P, Ch, B, Bs, acc, cpc);
-    } else {
-        if ((e = allow(k_up_umma<false>, smem)) != cudaSuccess) return e;
-        k_up_umma<false><<<grid, 128, smem, s>>>(P, Ch, B, Bs, acc, cpc);
-    }
-    return cudaGetLastError();
+    auto go = [&](auto kernel, int threads) -> cudaError_t {
+        if (cudaError_t e = allow(kernel, smem)) return e;
+        kernel<<<grid, threads, smem, s>>>(P, Ch, B, Bs, acc, cpc);
+        return cudaGetLastError();
+    };
+    if (smem <= (size_t)74 * 1024) return split ? go(k_up_umma<true, 128>, 128) : go(k_up_umma<false, 128>, 128);   // three CTAs per SM
+    return split ? go(k_up_umma<true, 256>, 256) : go(k_up_umma<false, 256>, 256);
 }
 
 // Tensor-core down pass from level l (P) into level l+1 (Ch), added into the
@@ -641,10 +654,10 @@ cudaError_t launch_down_umma(const DevLevel<float> &P, const DevLevel<float> &Ch
     cudaError_t e;
     if (split) {
         if ((e = allow(k_down_umma<true>, smem)) != cudaSuccess) return e;
-        k_down_umma<true><<<grid, 128, smem, s>>>(P, Ch, B, Bs, cpc, nbuf);
+        k_down_umma<true><<<grid, 256, smem, s>>>(P, Ch, B, Bs, cpc, nbuf);
     } else {
         if ((e = allow(k_down_umma<false>, smem)) != cudaSuccess) return e;
-        k_down_umma<false><<<grid, 128, smem, s>>>(P, Ch, B, Bs, cpc, nbuf);
+        k_down_umma<false><<<grid, 256, smem, s>>>(P, Ch, B, Bs, cpc, nbuf);
     }
     return cudaGetLastError();
 }
