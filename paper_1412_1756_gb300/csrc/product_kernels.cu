@@ -364,6 +364,8 @@ __global__ void __launch_bounds__(256) k_radiate(const int32_t *__restrict__ box
     }
 }
 
+constexpr int kMaxTypes = 343;   // translation types of one parent: offsets of a 7 x 7 x 7 cube at most
+
 // ---------------------------------------------------------- translate ---
 // Eq. (8) sample by sample, grouped by parent: the children of one parent
 // draw on one candidate set (children of the parent's neighbours), so each
@@ -391,19 +393,23 @@ __global__ void __launch_bounds__(128) k_translate(DevLevel<R> lv, int B, int Bs
     const int outs = blockDim.x / ES;
     const int q_lo = (blockIdx.y * outs) / BC;
     const int NQ = min(K - 1, (blockIdx.y * outs + outs - 1) / BC) - q_lo + 1;
-    if (SA) {
-        const int l0 = lv.lty_ptr[P], nl = lv.lty_ptr[P + 1] - l0;
-        const C *al = reinterpret_cast<const C *>(lv.alpha);
-        for (int i = threadIdx.x; i < nl * NQ; i += blockDim.x) {
-            const int lt = i / NQ, qq = i - lt * NQ;
-            cp_async(s_al + i, al + (int64_t)lv.lty[l0 + lt] * K + q_lo + qq);
-        }
-        cp_async_commit();
-    }
     const int16_t *tysrc = SA ? lv.grp_lty : lv.grp_ty;
     for (int e = threadIdx.x; e < ne; e += blockDim.x) s_src[e] = lv.grp_src[e0 + e];
     for (int e = threadIdx.x; e < ne * 8; e += blockDim.x) s_ty[e] = tysrc[(int64_t)e0 * 8 + e];
-    if (SA) cp_async_wait<0>();
+    if (SA) {
+        // the type list first: with its loads between the copies, each copy waited for one
+        __shared__ int s_lty[SA ? kMaxTypes : 1];
+        const int l0 = lv.lty_ptr[P], nl = lv.lty_ptr[P + 1] - l0;
+        for (int i = threadIdx.x; i < nl; i += blockDim.x) s_lty[i] = lv.lty[l0 + i];
+        __syncthreads();
+        const C *al = reinterpret_cast<const C *>(lv.alpha);
+        for (int i = threadIdx.x; i < nl * NQ; i += blockDim.x) {
+            const int lt = i / NQ, qq = i - lt * NQ;
+            cp_async(s_al + i, al + (int64_t)s_lty[lt] * K + q_lo + qq);
+        }
+        cp_async_commit();
+        cp_async_wait<0>();
+    }
     __syncthreads();
     const int part = threadIdx.x % ES;
     const int t = blockIdx.y * outs + threadIdx.x / ES;
@@ -1692,7 +1698,7 @@ cudaError_t launch_translate_es(const DevLevel<R> &Lv, int B, int Bs, int acc, c
     // samples one CTA touches, at most (its outputs may straddle a sample)
     const int nq = std::min(Lv.K, (128 / ES - 1) / (B / CB) + 2);
     const size_t smem = (size_t)Lv.max_lty * nq * sizeof(C);
-    if (Lv.lty && smem <= (size_t)48 * 1024)
+    if (Lv.lty && Lv.max_lty <= kMaxTypes && smem <= (size_t)40 * 1024)
         k_translate<R, ES, CB, true><<<grid, 128, smem, s>>>(Lv, B, Bs, acc);
     else
         k_translate<R, ES, CB, false><<<grid, 128, 0, s>>>(Lv, B, Bs, acc);
