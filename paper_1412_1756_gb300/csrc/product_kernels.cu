@@ -1438,6 +1438,11 @@ cudaError_t launch_near_wide(const ProductArgs<R> &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// Leaf boxes from which on two and three FP32 columns gain from the register
+// tiles of the near field and radiation (2 columns, us: 272 boxes 16 -> 26 and
+// 12 -> 17, 1,160 boxes 44 -> 40 and 38 -> 29).
+constexpr int kManyBoxes = 608;
+
 // Leaf boxes too few to give every SM two CTAs at one per box and 16 columns.
 bool few_boxes(int64_t boxes, int B) { return boxes * ((B + 15) / 16) < 2 * 152; }
 
@@ -1449,9 +1454,9 @@ cudaError_t launch_near(const ProductArgs<R> &a, cudaStream_t s, int choice = 0)
     if (choice == 1) return wide_ok ? launch_near_wide<R, 8>(a, s) : cudaErrorInvalidConfiguration;
     if (choice == 2) return wide_ok ? launch_near_wide<R, 16>(a, s) : cudaErrorInvalidConfiguration;
     if (choice == 3) return a.B >= 16 ? launch_near_bt<R, 16>(a, s) : cudaErrorInvalidConfiguration;
-    // register tiles: FP32 from two columns up; FP64, which its arithmetic bounds, where the tree has too few
+    // register tiles: FP32 from four columns up, from two on trees of many boxes; FP64, which its arithmetic bounds, where the tree has too few
     // leaf boxes to fill the GPU with one CTA per box (near_tile.cu has the figures of both sides)
-    if (sizeof(R) == 4 ? a.B >= 2 : (a.B >= 4 && few_boxes(a.nr.nleaf, a.B))) {
+    if (sizeof(R) == 4 ? (a.B >= 4 || (a.B >= 2 && a.nr.nleaf >= kManyBoxes)) : (a.B >= 4 && few_boxes(a.nr.nleaf, a.B))) {
         const cudaError_t e = launch_near_tile<R>(a, s);
         if (e != cudaErrorInvalidConfiguration) return e;
     }
@@ -1499,7 +1504,7 @@ cudaError_t launch_radiate(const ProductArgs<R> &a, int Bs, cudaStream_t s, int 
         }
     }
     // register tiles that follow the columns (leaf_tile.cu has the figures of both sides)
-    if (choice == 0 && (sizeof(R) == 4 ? a.B >= 2 : (a.B >= 4 && few_boxes(Lf.nbox, a.B)))) {
+    if (choice == 0 && (sizeof(R) == 4 ? (a.B >= 4 || (a.B >= 2 && Lf.nbox >= kManyBoxes)) : (a.B >= 4 && few_boxes(Lf.nbox, a.B)))) {
         const cudaError_t e = launch_radiate_tile<R>(a, Bs, s);
         if (e != cudaErrorInvalidConfiguration) return e;
     }

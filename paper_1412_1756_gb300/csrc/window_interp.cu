@@ -708,12 +708,15 @@ constexpr size_t kThird = 74 * 1024;   // down pass: shared memory for three CTA
 // against 1,857).  One or two columns take 2 per CTA (30,720-unknown sphere,
 // 2 columns: down from level 3 39 -> 35 us, up 53 -> 51 with 4 per CTA before;
 // 1 column, against the kernel of one row per thread: up 63 -> 51), except on
-// levels of a few boxes, whose few CTAs make a long chain (16 parents, 27 x
-// 54 samples, 2 columns: 16 us by the one-row kernel, 20 by this).
+// levels of few samples in all, whose few CTAs make a long chain (16 parents,
+// 27 x 54 samples, 2 columns: 16 us by the one-row kernel, 20 by this; 56
+// parents, 14 x 28 samples, 1 column: 22 against 25; 56 parents, 21 x 42:
+// 35 against 31).
+constexpr int64_t kFewSamples = 32 * 1024;
 template <bool PAIR>
 cudaError_t down_win_auto(const DevLevel<float> &P, const DevLevel<float> &Ch, int B, int Bs, cudaStream_t s)
 {
-    if (B <= 2 && Ch.nbox < 64) return cudaErrorInvalidConfiguration;   // left to the one-row kernel
+    if (B <= 2 && (int64_t)Ch.nbox * Ch.K < kFewSamples) return cudaErrorInvalidConfiguration;   // left to the one-row kernel
     if (B <= 2 && down_win_smem(P, Ch, 2) <= kThird) return down_win_nb<2, 3, PAIR>(P, Ch, B, Bs, s);
     if (!narrow_chunks(B) && down_win_smem(P, Ch, 8) <= kThird) return down_win_nb<8, 3, PAIR>(P, Ch, B, Bs, s);
     if (down_win_smem(P, Ch, 4) <= kThird) return down_win_nb<4, 3, PAIR>(P, Ch, B, Bs, s);
@@ -723,7 +726,7 @@ cudaError_t down_win_auto(const DevLevel<float> &P, const DevLevel<float> &Ch, i
 template <bool PAIR>
 cudaError_t up_win_auto(const DevLevel<float> &P, const DevLevel<float> &Ch, int B, int Bs, int acc, cudaStream_t s)
 {
-    if (B <= 2 && P.nbox < 32) return cudaErrorInvalidConfiguration;   // left to the one-row kernel
+    if (B <= 2 && (int64_t)P.nbox * P.K < kFewSamples) return cudaErrorInvalidConfiguration;   // left to the one-row kernel
     if (B <= 2 && up_win_smem(P, Ch, 2, 1) <= kUpCap3) return up_win_nb<2, 3, PAIR>(P, Ch, B, Bs, acc, s);
     if (!narrow_chunks(B)) {
         const size_t whole = up_win_smem(P, Ch, 8, 1);
