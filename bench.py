@@ -158,15 +158,18 @@ def fp32_peak_tflops(sm_mhz):
     return sm_count() * 128 * 2 * sm_mhz * 1e6 / 1e12
 
 
+# the product's kernels and their launchers
+PRODUCT_SOURCES = ("device.h", "product_kernels.cu", "window_interp.cu", "translate_quad.cu", "leaf_pairs.cu",
+                   "leaf_tile.cu", "near_tile.cu", "umma_interp.cu")
+
+
 def kernel_digest():
     """Digest of the product kernels' source: a DRAM-traffic figure taken by
     ncu is reported only while the kernels are the ones it was taken on."""
     import hashlib
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1412_1756_gb300", "csrc")
-    # the product's kernels and their launchers
-    for f in ("device.h", "product_kernels.cu", "window_interp.cu", "translate_quad.cu", "leaf_pairs.cu",
-              "umma_interp.cu"):
+    for f in PRODUCT_SOURCES:
         with open(os.path.join(csrc, f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
