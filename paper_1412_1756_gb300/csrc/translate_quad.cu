@@ -98,7 +98,8 @@ __global__ void __launch_bounds__(kThreads, MINB) k_translate_q4(DevLevel<float>
     __shared__ __align__(16) uint16_t s_ty[kMaxEntries * 8];   // per (entry, child): its row of the coefficients, or kNone
     const int K = lv.K;
     const int64_t KB = (int64_t)K * Bs;
-    const int P = blockIdx.x, i0 = blockIdx.y * kThreads;
+    const int P = blockIdx.x, i0 = (blockIdx.z * gridDim.y + blockIdx.y) * kThreads;
+    if (i0 >= K * nqd) return;   // of the last z slice
     const int q0 = i0 / nqd, nq = min(K, (i0 + kThreads - 1) / nqd + 1) - q0;   // nq <= QS
     const int e0 = lv.grp_ptr[P], ne = lv.grp_ptr[P + 1] - e0;
     const int m0 = lv.pchild_ptr[P], nc = lv.pchild_ptr[P + 1] - m0;
@@ -189,7 +190,11 @@ __global__ void __launch_bounds__(kThreads, MINB) k_translate_q4(DevLevel<float>
 template <bool FULL, bool PRE, int MINB>
 cudaError_t go(const DevLevel<float> &lv, int B, int Bs, int acc, int nqd, int QS, size_t smem, cudaStream_t s)
 {
-    dim3 grid(lv.nparent, (unsigned)(((int64_t)lv.K * nqd + kThreads - 1) / kThreads));
+    // a level of 8,192 samples (a body of 19 wavelengths) at 4,096 columns has 65,536 chunks of items, one more than
+    // grid.y takes: slices of equal size in z
+    const int64_t chunks = ((int64_t)lv.K * nqd + kThreads - 1) / kThreads, nz = (chunks + 65534) / 65535;
+    if (lv.K > (1 << 30) / nqd) return cudaErrorInvalidConfiguration;   // 32-bit item numbers (nz <= 129)
+    const dim3 grid(lv.nparent, (unsigned)((chunks + nz - 1) / nz), (unsigned)nz);
     k_translate_q4<FULL, PRE, MINB><<<grid, kThreads, smem, s>>>(lv, B, Bs, acc, nqd, QS);
     return cudaGetLastError();
 }
