@@ -26,7 +26,13 @@
 // field loads and four pattern loads feed 64 or 128 multiply-adds.  With few
 // columns (below 16) the threads left over after the tiles split the samples
 // (KS ways) and the partial sums are added in a fixed order; otherwise every
-// sum runs over the samples in order.  The field tile is requested one tile
+// sum runs over the samples in order.  In FP32 the samples of a tile (two
+// samples with 16 columns and more) are added up first and then join the
+// running sum: chained into it, four roundings per sample are of the running
+// sum's size, and five digits magnify them 700-fold (30,720-unknown sphere,
+// error against FP64 4.7e-5 at 8 columns, 6.8e-5 at 15, 4.5e-5 at 17; so
+// 3.6e-5, 3.9e-5, 3.5e-5, where k_receive_tiled with one rounding per sample
+// has 3.6e-5; reception takes 0-8 % longer).  The field tile is requested one tile
 // ahead and scaled by w_q on its way to shared memory, the patterns arrive
 // by cp.async one tile ahead.  Bound: instruction issue.  Measured, before ->
 // this (FP32, us): 30,720-unknown sphere 2 columns 47 -> 35, 10 columns 117
@@ -39,6 +45,7 @@
 #include "device.h"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace mlfma {
 
@@ -199,6 +206,20 @@ __device__ __forceinline__ void cmacc(R (&acc)[2], R vx, R vy, R gx, R gy)
     acc[1] = fma(vx, gy, fma(-vy, gx, acc[1]));
 }
 
+// acc += the sum over NS samples of both components' conj(v) * g
+template <class R, int NS>
+__device__ __forceinline__ void samples_acc(R (&acc)[2], const Four<R> (&v)[NS], const R (&g0)[NS][2], const R (&g1)[NS][2])
+{
+    R t[2] = {R(0), R(0)};
+#pragma unroll
+    for (int n = 0; n < NS; ++n) {
+        cmacc(t, v[n].x, v[n].y, g0[n][0], g0[n][1]);
+        cmacc(t, v[n].z, v[n].w, g1[n][0], g1[n][1]);
+    }
+    acc[0] += t[0];
+    acc[1] += t[1];
+}
+
 // CW columns of the field per thread
 template <class R, int CW> struct alignas(CW * 2 * sizeof(R) >= 16 ? 16 : CW * 2 * sizeof(R)) Cols { R v[2 * CW]; };
 
@@ -212,6 +233,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && CPT == 1 ? 3 : (sizeof(
 {
     using C = typename Cplx<R>::T;
     using G1 = Cols<R, CW>;
+    // acc is one tile's sum, tot the running sum
+    constexpr bool TS = sizeof(R) == 4 && CPT == 1;
     constexpr int VP = QT + 1;   // pitch of a staged pattern row: the rows a warp reads fall in different banks
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int GT = 2 * QT * ncp;                            // field tile: [component][sample][column group]
@@ -285,6 +308,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && CPT == 1 ? 3 : (sizeof(
             for (int k = 0; k < kRows; ++k)
 #pragma unroll
                 for (int c = 0; c < CW; ++c) acc[u][k][c][0] = acc[u][k][c][1] = R(0);
+        R tot[TS ? kRows : 1][CW][2] = {};
         {
             G1 g[NE];
             R w[NE];
@@ -305,31 +329,78 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && CPT == 1 ? 3 : (sizeof(
             if (ks < KS) {
                 const G1 *gs = Gs + (size_t)buf * GT + cp, *gs2 = gs + QT * ncp;
                 const Four<R> *vs = Vs + (size_t)buf * RP * VP + rg * VP;   // rows past the last: stale values, dropped
+                if constexpr (CPT == 1) {
 #pragma unroll 2
-                for (int qx = ks; qx < nq; qx += KS) {
-                    G1 g0[CPT], g1[CPT];
+                    for (int qx = ks; qx < nq; qx += KS) {
+                        const G1 g0 = gs[qx * ncp], g1 = gs2[qx * ncp];
 #pragma unroll
-                    for (int u = 0; u < CPT; ++u) {
-                        g0[u] = gs[qx * ncp + u * nct];
-                        g1[u] = gs2[qx * ncp + u * nct];
-                    }
+                        for (int k = 0; k < kRows; ++k) {
+                            const Four<R> v = vs[k * nrg * VP + qx];
 #pragma unroll
-                    for (int k = 0; k < kRows; ++k) {
-                        const Four<R> v = vs[k * nrg * VP + qx];
+                            for (int c = 0; c < CW; ++c) cmacc(acc[0][k][c], v.x, v.y, g0.v[2 * c], g0.v[2 * c + 1]);
 #pragma unroll
-                        for (int u = 0; u < CPT; ++u) {
-#pragma unroll
-                            for (int c = 0; c < CW; ++c) cmacc(acc[u][k][c], v.x, v.y, g0[u].v[2 * c], g0[u].v[2 * c + 1]);
-#pragma unroll
-                            for (int c = 0; c < CW; ++c) cmacc(acc[u][k][c], v.z, v.w, g1[u].v[2 * c], g1[u].v[2 * c + 1]);
+                            for (int c = 0; c < CW; ++c) cmacc(acc[0][k][c], v.z, v.w, g1.v[2 * c], g1.v[2 * c + 1]);
                         }
                     }
+                    if (TS) {
+#pragma unroll
+                        for (int k = 0; k < kRows; ++k)
+#pragma unroll
+                            for (int c = 0; c < CW; ++c)
+#pragma unroll
+                                for (int h = 0; h < 2; ++h) {
+                                    tot[k][c][h] += acc[0][k][c][h];
+                                    acc[0][k][c][h] = R(0);
+                                }
+                    }
+                } else {
+                    auto step = [&](int qx, auto ns) {
+                        constexpr int NS = decltype(ns)::value;
+                        G1 g0[NS][CPT], g1[NS][CPT];
+#pragma unroll
+                        for (int n = 0; n < NS; ++n)
+#pragma unroll
+                            for (int u = 0; u < CPT; ++u) {
+                                g0[n][u] = gs[(qx + n) * ncp + u * nct];
+                                g1[n][u] = gs2[(qx + n) * ncp + u * nct];
+                            }
+#pragma unroll
+                        for (int k = 0; k < kRows; ++k) {
+                            Four<R> v[NS];
+#pragma unroll
+                            for (int n = 0; n < NS; ++n) v[n] = vs[k * nrg * VP + qx + n];
+#pragma unroll
+                            for (int u = 0; u < CPT; ++u)
+#pragma unroll
+                                for (int c = 0; c < CW; ++c) {
+                                    R a0[NS][2], a1[NS][2];
+#pragma unroll
+                                    for (int n = 0; n < NS; ++n)
+#pragma unroll
+                                        for (int h = 0; h < 2; ++h) {
+                                            a0[n][h] = g0[n][u].v[2 * c + h];
+                                            a1[n][h] = g1[n][u].v[2 * c + h];
+                                        }
+                                    samples_acc<R, NS>(acc[u][k][c], v, a0, a1);
+                                }
+                        }
+                    };
+                    int qx = 0;   // KS = 1
+                    for (; qx + 1 < nq; qx += 2) step(qx, std::integral_constant<int, 2>{});
+                    if (qx < nq) step(qx, std::integral_constant<int, 1>{});
                 }
             }
             if (tile + 1 < ntile) store_g(buf ^ 1, g, w);
             wait_all_l();
             __syncthreads();   // the next tile is in; everyone is done with this one
         }
+        if (TS)
+#pragma unroll
+            for (int k = 0; k < kRows; ++k)
+#pragma unroll
+                for (int c = 0; c < CW; ++c)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) acc[0][k][c][h] = tot[k][c][h];
         auto add = [&](int r, int b, C s) {
             if (r < rows && b < nb) {
                 C *y = yp + (int64_t)(i0 + rp + r) * B + b0 + b;
@@ -345,7 +416,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && CPT == 1 ? 3 : (sizeof(
 #pragma unroll
                         for (int c = 0; c < CW; ++c)
                             add(rg + k * nrg, CW * (cp + u * nct) + c, C{acc[u][k][c][0], acc[u][k][c][1]});
-        } else if constexpr (CPT == 1) {   // the sample splits' partial sums, added in order of ks, one output per thread
+        } else if constexpr (CPT == 1) {   // the sample splits' partial sums, one output per thread
             C *part = reinterpret_cast<C *>(smem_raw);   // [KS][kRows][CW][tiles]
             const int outs = kRows * CW * tiles;
             if (ks < KS)
@@ -355,13 +426,24 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && CPT == 1 ? 3 : (sizeof(
                     for (int c = 0; c < CW; ++c) part[ks * outs + (k * CW + c) * tiles + tile_id] = C{acc[0][k][c][0], acc[0][k][c][1]};
             __syncthreads();
             for (int e = t; e < outs; e += nt) {
-                C s = part[e];
-#pragma unroll 4
-                for (int g = 1; g < KS; ++g) {
-                    const C w = part[g * outs + e];
-                    s.x += w.x;
-                    s.y += w.y;
-                }
+                const int n = min(KS, QT);   // the others had no sample
+                C p[4] = {};                 // in four chains: one of n terms rounds more often
+#pragma unroll 2
+                for (int g = 0; g + 3 < n; g += 4)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const C w = part[(g + j) * outs + e];
+                        p[j].x += w.x;
+                        p[j].y += w.y;
+                    }
+#pragma unroll
+                for (int j = 0; j < 3; ++j)
+                    if (j < (n & 3)) {
+                        const C w = part[((n & ~3) + j) * outs + e];
+                        p[j].x += w.x;
+                        p[j].y += w.y;
+                    }
+                const C s{(p[0].x + p[1].x) + (p[2].x + p[3].x), (p[0].y + p[1].y) + (p[2].y + p[3].y)};
                 const int kc = e / tiles, te = e - kc * tiles, k = kc / CW, c = kc - k * CW, r = te / ncp;
                 add(r + k * nrg, (te - r * ncp) * CW + c, s);
             }

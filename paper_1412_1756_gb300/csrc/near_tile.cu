@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kNT, sizeof(R) == 4 ? 3 : 2) k_near_tile(DevNe
                 for (int i = 0; i < kRT; ++i)
 #pragma unroll
                     for (int j = 0; j < CT; ++j) put(rg + i * nrg, cg * CT + j, acc[i][j]);
-        } else {   // the column splits' partial sums, added in order of ks, one output per thread
+        } else {   // the column splits' partial sums, one output per thread
             C *part = reinterpret_cast<C *>(smem_raw);   // [KS][kRT][CT][tiles]
             const int outs = kRT * CT * tiles;
             if (ks < KS)
@@ -175,13 +175,24 @@ __global__ void __launch_bounds__(kNT, sizeof(R) == 4 ? 3 : 2) k_near_tile(DevNe
                     for (int j = 0; j < CT; ++j) part[ks * outs + (i * CT + j) * tiles + tile] = acc[i][j];   // KS > 1 only in the last pass
             __syncthreads();
             for (int e = t; e < outs; e += kNT) {
-                C s = part[e];
-#pragma unroll 4
-                for (int g = 1; g < KS; ++g) {
-                    const C w = part[g * outs + e];
-                    s.x += w.x;
-                    s.y += w.y;
-                }
+                const int n = min(KS, KC);   // the others had no column
+                C p[4] = {};                 // in four chains: one of n terms rounds more often
+#pragma unroll 2
+                for (int g = 0; g + 3 < n; g += 4)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const C w = part[(g + j) * outs + e];
+                        p[j].x += w.x;
+                        p[j].y += w.y;
+                    }
+#pragma unroll
+                for (int j = 0; j < 3; ++j)
+                    if (j < (n & 3)) {
+                        const C w = part[((n & ~3) + j) * outs + e];
+                        p[j].x += w.x;
+                        p[j].y += w.y;
+                    }
+                const C s{(p[0].x + p[1].x) + (p[2].x + p[3].x), (p[0].y + p[1].y) + (p[2].y + p[3].y)};
                 const int ij = e / tiles, te = e - ij * tiles, i = ij / CT, j = ij - i * CT, r = te / ncg;
                 put(r + i * nrg, (te - r * ncg) * CT + j, s);
             }

@@ -1082,6 +1082,20 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && TM <= 20) ? 2 : 1)
     }
 }
 
+// acc += both components' conj(v) * g of one sample
+template <class C, class C4>
+__device__ __forceinline__ void sample_acc(C &acc, const C4 &v, const C &g0, const C &g1)
+{
+    C t{0, 0};
+    C &a = sizeof(C) == 8 ? t : acc;   // FP32: the sample's sum first, as leaf_tile.cu does and for its reason
+    cfmac(a, C{v.x, v.y}, g0);
+    cfmac(a, C{v.z, v.w}, g1);
+    if (sizeof(C) == 8) {
+        acc.x += t.x;
+        acc.y += t.y;
+    }
+}
+
 // ------------------------------------------------------------ receive ---
 // y_i += sum_q wq_q conj(V_s,mi(q)) . G_m(q).
 // Few columns: one CTA per (leaf box, chunk of LB columns) with the box's G
@@ -1135,10 +1149,8 @@ __global__ void __launch_bounds__(256) k_receive(const int32_t *__restrict__ box
             for (int q = lq; q < K; q += LQ) {
                 const C4 va = v[q], vc = v[K + q];
                 const C g0 = Gs[q * LB + lb], g1 = Gs[(K + q) * LB + lb];
-                cfmac(a, C{va.x, va.y}, g0);
-                cfmac(c, C{vc.x, vc.y}, g0);
-                cfmac(a, C{va.z, va.w}, g1);
-                cfmac(c, C{vc.z, vc.w}, g1);
+                sample_acc(a, va, g0, g1);
+                sample_acc(c, vc, g0, g1);
             }
             const bool upper = lane & 16;   // the upper half of the lanes goes on with the second unknown
             const R sx = upper ? a.x : c.x, sy = upper ? a.y : c.y;
@@ -1148,8 +1160,7 @@ __global__ void __launch_bounds__(256) k_receive(const int32_t *__restrict__ box
 #pragma unroll 4
             for (int q = lq; q < K; q += LQ) {
                 const C4 va = v[q];
-                cfmac(a, C{va.x, va.y}, Gs[q * LB + lb]);
-                cfmac(a, C{va.z, va.w}, Gs[(K + q) * LB + lb]);
+                sample_acc(a, va, Gs[q * LB + lb], Gs[(K + q) * LB + lb]);
             }
             a.x += __shfl_xor_sync(0xffffffffu, a.x, 16);
             a.y += __shfl_xor_sync(0xffffffffu, a.y, 16);
