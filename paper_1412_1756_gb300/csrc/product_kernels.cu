@@ -391,8 +391,9 @@ __global__ void __launch_bounds__(128) k_translate(DevLevel<R> lv, int B, int Bs
     const int K = lv.K;
     const int BC = B / CB;                 // column groups (B is a multiple of CB)
     const int outs = blockDim.x / ES;
-    const int q_lo = (blockIdx.y * outs) / BC;
-    const int NQ = min(K - 1, (blockIdx.y * outs + outs - 1) / BC) - q_lo + 1;
+    const int by = ES > 1 ? blockIdx.y : blockIdx.z * 65535 + blockIdx.y;   // z: slices of long bodies
+    const int q_lo = (by * outs) / BC;
+    const int NQ = min(K - 1, (by * outs + outs - 1) / BC) - q_lo + 1;
     const int16_t *tysrc = SA ? lv.grp_lty : lv.grp_ty;
     for (int e = threadIdx.x; e < ne; e += blockDim.x) s_src[e] = lv.grp_src[e0 + e];
     for (int e = threadIdx.x; e < ne * 8; e += blockDim.x) s_ty[e] = tysrc[(int64_t)e0 * 8 + e];
@@ -412,7 +413,7 @@ __global__ void __launch_bounds__(128) k_translate(DevLevel<R> lv, int B, int Bs
     }
     __syncthreads();
     const int part = threadIdx.x % ES;
-    const int t = blockIdx.y * outs + threadIdx.x / ES;
+    const int t = by * outs + threadIdx.x / ES;
     const bool valid = t < K * BC;
     const int q = valid ? t / BC : 0, b = valid ? (t % BC) * CB : 0;
     const C *S = reinterpret_cast<const C *>(lv.S);
@@ -1709,8 +1710,10 @@ template <class R, int ES, int CB>
 cudaError_t launch_translate_es(const DevLevel<R> &Lv, int B, int Bs, int acc, cudaStream_t s)
 {
     using C = typename Cx<R>::T;
-    const int outs = Lv.K * (B / CB);
-    dim3 grid(Lv.nparent, (outs + 128 / ES - 1) / (128 / ES));
+    if (Lv.K > (1 << 30) / (B / CB)) return cudaErrorInvalidConfiguration;   // 32-bit output numbers
+    const int ctas = (Lv.K * (B / CB) + 128 / ES - 1) / (128 / ES), nz = (ctas + 65534) / 65535;   // grid.y holds 65,535
+    if (ES > 1 && nz > 1) return cudaErrorInvalidConfiguration;   // lanes share outputs only where there are few
+    const dim3 grid(Lv.nparent, std::min(ctas, 65535), nz);
     // samples one CTA touches, at most (its outputs may straddle a sample)
     const int nq = std::min(Lv.K, (128 / ES - 1) / (B / CB) + 2);
     const size_t smem = (size_t)Lv.max_lty * nq * sizeof(C);

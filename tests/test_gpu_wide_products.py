@@ -1,9 +1,10 @@
 """Products of many columns on long thin bodies: the samples of a coarse level
 times the columns exceed what one further grid dimension can count (65,535
-CTAs of 128 items), in the built-in translation of FP32 fields.  Checked
-against products of 16 of the same columns.  Tolerance (relative 2-norm, fixed
-from the arithmetic): FP32 rounding magnified by the growth of the Hankel
-terms, |h_L(kr)| up to ~70 for three digits, 1e-4."""
+CTAs of 128 items), in the built-in translations of FP32 and of FP64 fields.
+Checked against products of 16 of the same columns.  Tolerances (relative
+2-norm, fixed from the arithmetic): FP32 rounding magnified by the growth of
+the Hankel terms, |h_L(kr)| up to ~70 for three digits, 1e-4; FP64 sums in
+another order 1e-10."""
 import numpy as np
 import pytest
 
@@ -19,6 +20,7 @@ K = 2 * np.pi
 
 @pytest.mark.parametrize("length,levels,per_item,dt,tol", [
     (19.2, 7, 4, torch.float32, 1e-4),     # 9,248 samples at level 2, four columns per item
+    (12.8, 6, 2, torch.float64, 1e-10),    # 4,802 samples, two columns per thread
 ])
 def test_translation_grid_of_long_bodies(length, levels, per_item, dt, tol):
     v, t = workloads.plate(length, 0.2, int(round(10 * length)), 2)
