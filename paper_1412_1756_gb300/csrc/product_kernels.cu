@@ -364,8 +364,6 @@ __global__ void __launch_bounds__(256) k_radiate(const int32_t *__restrict__ box
     }
 }
 
-constexpr int kMaxTypes = 343;   // translation types of one parent: offsets of a 7 x 7 x 7 cube at most
-
 // ---------------------------------------------------------- translate ---
 // Eq. (8) sample by sample, grouped by parent: the children of one parent
 // draw on one candidate set (children of the parent's neighbours), so each
@@ -384,7 +382,8 @@ __global__ void __launch_bounds__(128) k_translate(DevLevel<R> lv, int B, int Bs
     __shared__ int s_src[216];
     __shared__ __align__(16) int16_t s_ty[216 * 8];
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *s_al = reinterpret_cast<C *>(smem_raw);   // SA: [local type][NQ]
+    // SA: the parent's local types, then (16-byte aligned) their coefficients [local type][NQ]
+    int *s_lty = reinterpret_cast<int *>(smem_raw);
     const int P = blockIdx.x;
     const int e0 = lv.grp_ptr[P], ne = lv.grp_ptr[P + 1] - e0;
     const int m0 = lv.pchild_ptr[P], nc = lv.pchild_ptr[P + 1] - m0;
@@ -392,15 +391,16 @@ __global__ void __launch_bounds__(128) k_translate(DevLevel<R> lv, int B, int Bs
     const int BC = B / CB;                 // column groups (B is a multiple of CB)
     const int outs = blockDim.x / ES;
     const int by = ES > 1 ? blockIdx.y : blockIdx.z * 65535 + blockIdx.y;   // z: slices of long bodies
+    if (ES == 1 && by * outs >= K * BC) return;                            // past the end of the last slice
     const int q_lo = (by * outs) / BC;
     const int NQ = min(K - 1, (by * outs + outs - 1) / BC) - q_lo + 1;
+    const int l0 = SA ? lv.lty_ptr[P] : 0, nl = SA ? lv.lty_ptr[P + 1] - l0 : 0;
+    C *s_al = reinterpret_cast<C *>(smem_raw + (nl + 3) / 4 * 16);
     const int16_t *tysrc = SA ? lv.grp_lty : lv.grp_ty;
     for (int e = threadIdx.x; e < ne; e += blockDim.x) s_src[e] = lv.grp_src[e0 + e];
     for (int e = threadIdx.x; e < ne * 8; e += blockDim.x) s_ty[e] = tysrc[(int64_t)e0 * 8 + e];
     if (SA) {
         // the type list first: with its loads between the copies, each copy waited for one
-        __shared__ int s_lty[SA ? kMaxTypes : 1];
-        const int l0 = lv.lty_ptr[P], nl = lv.lty_ptr[P + 1] - l0;
         for (int i = threadIdx.x; i < nl; i += blockDim.x) s_lty[i] = lv.lty[l0 + i];
         __syncthreads();
         const C *al = reinterpret_cast<const C *>(lv.alpha);
@@ -1716,9 +1716,13 @@ cudaError_t launch_translate_es(const DevLevel<R> &Lv, int B, int Bs, int acc, c
     const dim3 grid(Lv.nparent, std::min(ctas, 65535), nz);
     // samples one CTA touches, at most (its outputs may straddle a sample)
     const int nq = std::min(Lv.K, (128 / ES - 1) / (B / CB) + 2);
-    const size_t smem = (size_t)Lv.max_lty * nq * sizeof(C);
-    if (Lv.lty && Lv.max_lty <= kMaxTypes && smem <= (size_t)40 * 1024)
-        k_translate<R, ES, CB, true><<<grid, 128, smem, s>>>(Lv, B, Bs, acc);
+    // staged up to 48 KB, where four CTAs share an SM and it comes out even (41-48 KB, staged and not, us: FP64 7 columns
+    // of 7,680 unknowns 303 and 330, 6 columns of 7,200 354 and 340; FP32 122,880 unknowns, 3 columns 70 and 59, 6
+    // columns 77 and 94).  The list is as long as the level's largest: at its bound of 343 types it had cost the eighth
+    // CTA per SM (FP32 7 columns, 23 KB of coefficients, 292 against 244 at the leaf level of 122,880 unknowns).
+    const size_t coef = (size_t)Lv.max_lty * nq * sizeof(C);
+    if (Lv.lty && coef <= (size_t)48 * 1024)
+        k_translate<R, ES, CB, true><<<grid, 128, coef + (size_t)(Lv.max_lty + 3) / 4 * 16, s>>>(Lv, B, Bs, acc);
     else
         k_translate<R, ES, CB, false><<<grid, 128, 0, s>>>(Lv, B, Bs, acc);
     return cudaGetLastError();
@@ -1886,6 +1890,8 @@ cudaError_t prime_kernels()
     ALLOW((k_near<R, 8, true>)); ALLOW((k_near<R, 16, true>));
     ALLOW((k_near_wide<R, 8>)); ALLOW((k_near_wide<R, 16>));
     ALLOW((k_down_pp<R, 4, 16>)); ALLOW((k_down_pp<R, 4, 20>)); ALLOW((k_down_pp<R, 8, 16>)); ALLOW((k_down_pp<R, 8, 20>));
+    ALLOW((k_translate<R, 1, 2, true>)); ALLOW((k_translate<R, 1, 1, true>)); ALLOW((k_translate<R, 2, 1, true>));
+    ALLOW((k_translate<R, 4, 1, true>)); ALLOW((k_translate<R, 8, 1, true>)); ALLOW((k_translate<R, 16, 1, true>));
     ALLOW(k_radiate<R>);
     ALLOW(k_radiate_wide<R>);
     ALLOW((k_radiate_tiled<R, 8, 4>)); ALLOW((k_radiate_tiled<R, 16, 4>)); ALLOW((k_radiate_tiled<R, 32, 4>));
