@@ -229,7 +229,7 @@ template <class R, int CW> struct alignas(CW * 2 * sizeof(R) >= 16 ? 16 : CW * 2
 template <class R, int CW, int QT, int NE, int CPT>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 && CPT == 1 ? 3 : (sizeof(R) == 4 ? 2 : 1)) k_receive_tile(const int32_t *__restrict__ box_ptr, const Four<R> *__restrict__ V4,
                                                       DevLevel<R> lf, typename Cplx<R>::T *__restrict__ yp, int B, int Bs,
-                                                      int ncp, int RP, int split)
+                                                      int ncp, int RP)
 {
     using C = typename Cplx<R>::T;
     using G1 = Cols<R, CW>;
@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && CPT == 1 ? 3 : (sizeof(
     };
     for (int rp = ra; rp < rz; rp += RP) {
         const int rows = min(RP, rz - rp), nrg = (rows + kRows - 1) / kRows, nct = ncp / CPT, tiles = nrg * nct;
-        const int KS = split ? max(1, nt / tiles) : 1;
+        const int KS = CPT == 1 ? max(1, nt / tiles) : 1;
         const int ks = t / tiles, tile_id = t - ks * tiles, rg = tile_id / nct, cp = tile_id - rg * nct;
         auto stage_v = [&](int tile, int buf) {
             const int q0 = tile * QT, nq = K - q0;
@@ -480,28 +480,37 @@ cudaError_t radiate_go(const ProductArgs<R> &a, int Bs, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// Row groups of the usual leaf box, a quarter above the mean; larger boxes take more passes.
+template <class R>
+int usual_groups(const ProductArgs<R> &a, int nbox)
+{
+    const int mean = (int)(a.n / std::max(1, nbox)) + 1;
+    return (mean + mean / 4 + kRows - 1) / kRows;
+}
+
 template <class R, int CW, int QT, int NE, int CPT = 1>
 cudaError_t receive_go(const ProductArgs<R> &a, int Bs, int ncp, cudaStream_t s)
 {
     const DevLevel<R> &Lf = a.lv[a.leaf];
-    const int split = CPT == 1 && a.B < 16;   // few columns: the samples are split over the threads left over
+    constexpr bool split = CPT == 1;   // the samples are split over the threads left over
     const int nct = ncp / CPT;
-    // threads for the usual box (a quarter above the mean rows); larger boxes take more passes
-    const int mean = (int)(a.n / std::max(1, Lf.nbox)) + 1, want = (mean + mean / 4 + kRows - 1) / kRows;
-    const int least = (2 * QT * ncp + NE - 1) / NE;   // NE field elements per thread and tile
-    const int threads = split ? 256 : std::min(256, (std::max({64, nct * want, least}) + 31) / 32 * 32);
-    const int RP = std::min((a.nr.max_rows + kRows - 1) / kRows, threads / nct) * kRows;
+    const int64_t ctas = (int64_t)Lf.nbox * ((a.B + CW * ncp - 1) / (CW * ncp));
+    const int all = (a.nr.max_rows + kRows - 1) / kRows;   // row groups of the largest box
+    int rs = 1;   // row splits: fill the GPU when the tree has few leaf boxes
+    while (ctas * rs < 2 * 152 && 4 * rs * kRows <= a.nr.max_rows) rs *= 2;
+    const int least = std::max((2 * QT * ncp + NE - 1) / NE, 64);   // NE field elements per thread and tile
+    int threads = split ? 256 : std::min(256, (std::max(nct * usual_groups(a, Lf.nbox), least) + 31) / 32 * 32);
+    // a split needs fewer than the whole box: down to what runs in one wave (128 registers a thread)
+    while (!split && rs > 1 && ctas * rs > 152 * (512 / threads) && threads - 32 >= std::max(least, nct * ((all + rs - 1) / rs)))
+        threads -= 32;
+    const int RP = std::min(all, threads / nct) * kRows;
     if (2 * QT * ncp > NE * threads || (int64_t)2 * Lf.K * Bs > INT32_MAX) return cudaErrorInvalidConfiguration;   // 32-bit field offsets
     const size_t stage = (size_t)4 * QT * ncp * sizeof(Cols<R, CW>) + (size_t)2 * RP * (QT + 1) * sizeof(Four<R>);
     const size_t part = split ? (size_t)256 * kRows * CW * 2 * sizeof(R) : 0;
     const size_t smem = std::max(stage, part);
     if (smem > (size_t)kLeafSmem) return cudaErrorInvalidConfiguration;
-    const int64_t ctas = (int64_t)Lf.nbox * ((a.B + CW * ncp - 1) / (CW * ncp));
-    int rs = 1;   // row splits: fill the GPU when the tree has few leaf boxes
-    while (ctas * rs < 2 * 152 && 4 * rs * kRows <= a.nr.max_rows) rs *= 2;
     k_receive_tile<R, CW, QT, NE, CPT><<<dim3((unsigned)ctas, rs), threads, smem, s>>>(
-        a.nr.box_ptr, reinterpret_cast<const Four<R> *>(a.V), Lf, reinterpret_cast<typename Cplx<R>::T *>(a.yp), a.B, Bs, ncp, RP,
-        split);
+        a.nr.box_ptr, reinterpret_cast<const Four<R> *>(a.V), Lf, reinterpret_cast<typename Cplx<R>::T *>(a.yp), a.B, Bs, ncp, RP);
     return cudaGetLastError();
 }
 
@@ -524,6 +533,16 @@ cudaError_t launch_receive_tile(const ProductArgs<R> &a, int Bs, cudaStream_t s)
     if constexpr (sizeof(R) == 4) {
         if (ncp <= 4) return receive_go<R, 2, 32, 1>(a, Bs, ncp, s);
         if (ncp <= 8) return receive_go<R, 2, 16, 1>(a, Bs, ncp, s);
+        // From 17 columns up, k_receive_pairs (32 columns a CTA) where the tile's chunks of 64 leave a third of their
+        // columns empty (a remainder of 1-32, but for boxes of 96 rows and more), and where no column is empty in
+        // either (32, or a remainder of 61-64 on fewer than 4,096 boxes) but the tile's threads take the larger boxes
+        // in two passes.  Pairs / tile, us: 80 columns of 30,720 unknowns 350 / 459, of 7,680 139 / 217; 32
+        // columns of 30,720 145 / 174, of 115,200 708 / 804, of 42,960 (plate, one pass) 255 / 220; 64 columns of
+        // 28,800 391 / 422, of 115,200 1,302 / 1,277; 96 columns on boxes of 175 rows 406 / 270.
+        const int nct = std::min((ncp + 1) / 2, 16), rest = a.B % 64;
+        const bool passes = (a.nr.max_rows + kRows - 1) / kRows > std::max(64, (nct * usual_groups(a, a.lv[a.leaf].nbox) + 31) / 32 * 32) / nct;
+        const bool full = a.B == 32 || ((rest == 0 || rest > 60) && a.lv[a.leaf].nbox < 4096);
+        if ((a.B > 64 && rest > 0 && rest <= 32 && a.nr.max_rows < 96) || (full && passes)) return launch_receive_pairs(a, Bs, 32, s);
         return receive_go<R, 2, 8, 4, 2>(a, Bs, std::min((ncp + 1) / 2 * 2, 32), s);
     } else {
         return receive_go<R, 2, 16, 1>(a, Bs, std::min(ncp, 8), s);

@@ -1587,13 +1587,22 @@ cudaError_t launch_receive(const ProductArgs<R> &a, int Bs, cudaStream_t s, int 
         else return cudaErrorInvalidConfiguration;
     }
     if (choice == 0) {
-        // register tiles that follow the columns (leaf_tile.cu has the figures of both sides); one full chunk of 16
-        // is left to the 16-column kernel
-        if (sizeof(R) == 8 ? (a.B >= 5 || (a.B >= 3 && few_boxes(a.lv[a.leaf].nbox, a.B))) : (a.B >= 2 && a.B != 16)) {
+        // Register tiles that follow the columns (leaf_tile.cu has the figures of both sides).  FP32: from two columns up,
+        // but for one full chunk of 16 (61 us by the 16-column kernel, 76 by the tile, 10,824 unknowns).  FP64: where the
+        // tree has few leaf boxes from three columns up (1,920 unknowns, 4 columns 88 -> 49), else from five; seven are two
+        // chunks of four in k_receive (28,800 unknowns, 596 us for four columns, 1,420 for seven by the tile).  Boxes of
+        // fewer than 16 rows leave most of a tile's threads idle: only 2-15 columns in FP32 and 8-10 in FP64, where the
+        // threads just cover a tile's samples (480 unknowns, us: FP32 32 columns 24 older, 37 tile; FP64 4 columns 31 and 43,
+        // 8 columns 74 and 47, 12 columns 74 and 98).
+        const bool small = a.nr.max_rows < 16, few = few_boxes(a.lv[a.leaf].nbox, a.B);
+        if (sizeof(R) == 8 ? (small ? a.B >= 8 && a.B <= 10 : few ? a.B >= 3 : a.B >= 5 && a.B != 7)
+                           : (a.B >= 2 && (small ? a.B < 16 : a.B != 16))) {
             const cudaError_t e = launch_receive_tile<R>(a, Bs, s);
             if (e != cudaErrorInvalidConfiguration) return e;
         }
     }
+    if constexpr (sizeof(R) == 4)   // boxes of few rows
+        if (choice == 0 && a.B >= 32) return launch_receive_pairs(a, Bs, 32, s);
     if (choice == 1) return a.B >= 32 ? launch_receive_tiled<R, 32>(a, Bs, s) : cudaErrorInvalidConfiguration;
     if (choice == 2) return a.B >= 16 ? launch_receive_tiled<R, 16>(a, Bs, s) : cudaErrorInvalidConfiguration;
     if (choice == 3) return a.B >= 8 ? launch_receive_tiled<R, 8>(a, Bs, s) : cudaErrorInvalidConfiguration;
