@@ -687,9 +687,13 @@ bool win_ok(const WinDev &a, const WinDev &b) { return a.groups > 0 && b.groups 
 
 namespace {
 
-// Columns per CTA of the built-in choice: 8, or 4 where 8 would leave a
-// sixth of the chunks' columns empty.
-bool narrow_chunks(int B) { return 6 * ((B + 3) / 4 * 4) <= 5 * ((B + 7) / 8 * 8); }
+// Columns per CTA of the built-in choice: 8, or 4 where 8 would leave a fifth
+// of the chunks' columns empty, a sixth in the up pass with two CTAs per SM
+// (20 columns, 8 and 4 per CTA, us: down from 14 x 28 samples, 122,880
+// unknowns, 516 and 590, from 16 x 32, 115,200 unknowns, 713 and 755; up into
+// 14 x 28 547 and 585, into 16 x 32, two CTAs, 658 and 617; 12 columns, down
+// 348 and 358, up 374 and 357).
+bool narrow_chunks(int B, int empty = 5) { return empty * ((B + 3) / 4 * 4) <= (empty - 1) * ((B + 7) / 8 * 8); }
 
 constexpr size_t kThird = 74 * 1024;   // down pass: shared memory for three CTAs per SM
 
@@ -711,13 +715,24 @@ constexpr size_t kThird = 74 * 1024;   // down pass: shared memory for three CTA
 // levels of few samples in all, whose few CTAs make a long chain (16 parents,
 // 27 x 54 samples, 2 columns: 16 us by the one-row kernel, 20 by this; 56
 // parents, 14 x 28 samples, 1 column: 22 against 25; 56 parents, 21 x 42:
-// 35 against 31).
-constexpr int64_t kFewSamples = 32 * 1024;
+// 35 against 31).  One column leaves half of a CTA's columns empty, which the
+// one-row kernel does not: it keeps levels where two columns do not fit three
+// CTAs per SM (four per CTA had taken their place: up into 34 x 68 samples 61
+// against 55, down from 38 x 76 59 against 37), levels of many samples in all
+// (up into 1,160 boxes of 14 x 28 94 against 84, 1,160 of 17 x 34 117 against
+// 102; 272 of 27 x 54 78 against 87) and the down pass from fewer than 450
+// samples (1,160 pairs, 14 x 28, 111 against 102; 16 x 32 137 against 178).
+// Flat bodies have no children that share a phi step, so their up pass of one
+// or two columns stays with it too (plate of 12 wavelengths, 1 column: into 46
+// x 92 51 against 25, into 27 x 54 43 against 35).
+constexpr int64_t kFewSamples = 32 * 1024, kManySamples = 430 * 1024;
 template <bool PAIR>
 cudaError_t down_win_auto(const DevLevel<float> &P, const DevLevel<float> &Ch, int B, int Bs, cudaStream_t s)
 {
-    if (B <= 2 && (int64_t)Ch.nbox * Ch.K < kFewSamples) return cudaErrorInvalidConfiguration;   // left to the one-row kernel
-    if (B <= 2 && down_win_smem(P, Ch, 2) <= kThird) return down_win_nb<2, 3, PAIR>(P, Ch, B, Bs, s);
+    const bool two = down_win_smem(P, Ch, 2) <= kThird;
+    if ((B <= 2 && (int64_t)Ch.nbox * Ch.K < kFewSamples) || (B == 1 && (!two || P.K < 450)))
+        return cudaErrorInvalidConfiguration;   // left to the one-row kernel
+    if (B <= 2 && two) return down_win_nb<2, 3, PAIR>(P, Ch, B, Bs, s);
     if (!narrow_chunks(B) && down_win_smem(P, Ch, 8) <= kThird) return down_win_nb<8, 3, PAIR>(P, Ch, B, Bs, s);
     if (down_win_smem(P, Ch, 4) <= kThird) return down_win_nb<4, 3, PAIR>(P, Ch, B, Bs, s);
     return down_win_nb<4, 2, PAIR, 512>(P, Ch, B, Bs, s);
@@ -726,14 +741,21 @@ cudaError_t down_win_auto(const DevLevel<float> &P, const DevLevel<float> &Ch, i
 template <bool PAIR>
 cudaError_t up_win_auto(const DevLevel<float> &P, const DevLevel<float> &Ch, int B, int Bs, int acc, cudaStream_t s)
 {
-    if (B <= 2 && (int64_t)P.nbox * P.K < kFewSamples) return cudaErrorInvalidConfiguration;   // left to the one-row kernel
-    if (B <= 2 && up_win_smem(P, Ch, 2, 1) <= kUpCap3) return up_win_nb<2, 3, PAIR>(P, Ch, B, Bs, acc, s);
+    const int64_t samples = (int64_t)P.nbox * P.K;
+    const bool two = up_win_smem(P, Ch, 2, 1) <= kUpCap3, flat = PAIR && P.ndgrp == Ch.nbox;
+    if ((B <= 2 && (samples < kFewSamples || flat)) || (B == 1 && (!two || samples > kManySamples)))
+        return cudaErrorInvalidConfiguration;   // left to the one-row kernel
+    if (B <= 2 && two) return up_win_nb<2, 3, PAIR>(P, Ch, B, Bs, acc, s);
     if (!narrow_chunks(B)) {
         const size_t whole = up_win_smem(P, Ch, 8, 1);
         if (whole <= kUpCap3) return up_win_nb<8, 3, PAIR>(P, Ch, B, Bs, acc, s);
-        if (whole <= kUpCap2) return up_win_nb<8, 2, PAIR>(P, Ch, B, Bs, acc, s);
-        // too few parents to fill the GPU: bands cost nothing, and fewer, wider chunks load the children less often
-        if ((int64_t)P.nbox * 2 * ((B + 7) / 8) <= 2 * 152) return up_win_nb<8, 2, PAIR>(P, Ch, B, Bs, acc, s);
+        if (whole <= kUpCap2 && !narrow_chunks(B, 6)) return up_win_nb<8, 2, PAIR>(P, Ch, B, Bs, acc, s);
+        // too few parents to fill the GPU: bands cost nothing, and fewer, wider chunks load the children less often, as
+        // long as bands of one group are small beside the child's field, which every band loads (16 columns, 8 and 4 per
+        // CTA, us: 56 parents of 24 x 48 samples 68 and 80, 16 of 27 x 54 31 and 45; 56 of 34 x 68 174 and 141, 56 of
+        // 46 x 92 393 and 264)
+        if ((int64_t)P.nbox * 2 * ((B + 7) / 8) <= 2 * 152 && up_win_smem(P, Ch, 8, P.wu_th.groups) <= kUpCap3)
+            return up_win_nb<8, 2, PAIR>(P, Ch, B, Bs, acc, s);
     }
     if (up_win_smem(P, Ch, 4, 1) <= kUpCap3) return up_win_nb<4, 3, PAIR>(P, Ch, B, Bs, acc, s);
     return up_win_nb<4, 2, PAIR>(P, Ch, B, Bs, acc, s);
