@@ -462,16 +462,20 @@ template <class R, int CC>
 cudaError_t radiate_go(const ProductArgs<R> &a, int Bs, cudaStream_t s)
 {
     const DevLevel<R> &Lf = a.lv[a.leaf];
-    const int ncq = std::min((a.B + CC - 1) / CC, sizeof(R) == 4 ? 16 : 8);
-    int slots = std::max(1, std::min(256 / ncq, (Lf.K + 1) / 2));   // a thread's two samples are one slot
+    // column chunks and sample tiles of even size: 65 columns as 36 + 29 and not 64 + 1, 288 samples as 144 + 144 and not
+    // 256 + 32, whose last CTA or step leaves most threads idle
+    const int groups = (a.B + CC - 1) / CC, most = sizeof(R) == 4 ? 16 : 8, nch = (groups + most - 1) / most;
+    const int ncq = (groups + nch - 1) / nch;
     const int64_t ctas = (int64_t)Lf.nbox * ((a.B + CC * ncq - 1) / (CC * ncq));
+    int SL = std::max(1, std::min(256 / ncq, (Lf.K + 1) / 2));   // a thread's two samples are one slot
     // few leaf boxes: shorter sample tiles, so that their splits fill the GPU
-    while (slots * ncq > 32 && ctas * ((Lf.K + 2 * slots - 1) / (2 * slots)) < 2 * 152) slots = (slots + 1) / 2;
-    const int threads = std::min(256, (slots * ncq + 31) / 32 * 32), SL = std::min(threads / ncq, (Lf.K + 1) / 2);
-    const int QT = 2 * SL, RR = std::max(1, 1024 / QT);
+    while (SL * ncq > 32 && ctas * ((Lf.K + 2 * SL - 1) / (2 * SL)) < 2 * 152) SL = (SL + 1) / 2;
+    SL = std::min((SL * ncq + 31) / 32 * 32 / ncq, (Lf.K + 1) / 2);   // the last warp's threads
+    const int ntile = (Lf.K + 2 * SL - 1) / (2 * SL);
+    SL = (Lf.K + 2 * ntile - 1) / (2 * ntile);
+    const int threads = (SL * ncq + 31) / 32 * 32, QT = 2 * SL, RR = std::max(1, 1024 / QT);
     const size_t smem = (size_t)2 * RR * QT * sizeof(Four<R>) + (size_t)a.nr.max_rows * ncq * CC * sizeof(R);
     if (smem > (size_t)kLeafSmem) return cudaErrorInvalidConfiguration;
-    const int ntile = (Lf.K + QT - 1) / QT;
     int qs = 1;
     while (ctas * qs < 2 * 152 && qs < ntile) ++qs;
     k_radiate_tile<R, CC><<<dim3((unsigned)ctas, qs), threads, smem, s>>>(
