@@ -202,18 +202,27 @@ __global__ void __launch_bounds__(kNT, sizeof(R) == 4 ? 3 : 2) k_near_tile(DevNe
 }
 
 template <class R, int CT>
-cudaError_t go(const ProductArgs<R> &a, int nbc, cudaStream_t s)
+cudaError_t go(const ProductArgs<R> &a, int most, cudaStream_t s)
 {
     using C = typename Cplx<R>::T;
+    // a small remainder is shared out, 65 columns as 36 + 29 (30,720 unknowns: 245 us as 64 + 1, 228 so; 96 columns 245 as
+    // 64 + 32, 257 as 48 + 48)
+    const int chunks = (a.B + most - 1) / most, rest = a.B % most;
+    const int nbc = rest > 0 && 2 * rest < most ? ((a.B + chunks - 1) / chunks + CT - 1) / CT * CT : most;
     const int nch = (a.B + nbc - 1) / nbc, ncg = (std::min(a.B, nbc) + CT - 1) / CT, XP = ncg * CT;
-    // few columns: the strips stream past, so larger chunks keep more bytes in flight
-    const int KC = ncg <= 2 ? 64 : 32;
+    // few columns: the strips stream past, so larger chunks keep more bytes in flight; large boxes take what fits (boxes of
+    // 175 rows, FP64, 4 columns: 482 us with chunks of 32, 986 by the kernel of one row per thread; where 64 fit, 32 for
+    // the sake of more CTAs per SM lose, 120 against 105 us at 4 FP32 columns)
+    int KC = ncg <= 2 ? 64 : 32;
+    auto need = [&](int kc) {
+        const size_t z = (size_t)(kc * a.nr.max_rows + 8) / 2 * 2, x = (size_t)(kc * XP + 3) / 4 * 4;
+        // the column indices follow the staging buffers; the partial sums may run over them (they are used up by then)
+        return std::max(2 * z * sizeof(C) + 2 * x * sizeof(R) + (size_t)a.nr.max_cols * sizeof(int), (size_t)kNT * kRT * CT * sizeof(C));
+    };
+    while (KC > 16 && need(KC) > (size_t)kNearTileSmem) KC /= 2;
     const int zcap = (KC * a.nr.max_rows + 8) / 2 * 2;   // even, so the second buffer stays 16-byte aligned
     const int xcap = (KC * XP + 3) / 4 * 4;
-    const size_t stage = 2 * (size_t)zcap * sizeof(C) + 2 * (size_t)xcap * sizeof(R);
-    const size_t part = (size_t)kNT * kRT * CT * sizeof(C);
-    // the column indices follow the staging buffers; the partial sums may run over them (they are used up by then)
-    const size_t smem = std::max(stage + (size_t)a.nr.max_cols * sizeof(int), part);
+    const size_t smem = need(KC);
     if (smem > (size_t)kNearTileSmem) return cudaErrorInvalidConfiguration;
     // pieces of an x row: as wide as B, the chunk and the buffer's address allow
     const int chunk = std::min(a.B, nbc);

@@ -1452,8 +1452,10 @@ cudaError_t launch_near_wide(const ProductArgs<R> &a, cudaStream_t s)
 
 // Leaf boxes from which on two and three FP32 columns gain from the register
 // tiles of the near field and radiation (2 columns, us: 272 boxes 16 -> 26 and
-// 12 -> 17, 1,160 boxes 44 -> 40 and 38 -> 29).
-constexpr int kManyBoxes = 608;
+// 12 -> 17, 1,160 boxes 44 -> 40 and 38 -> 29), and from which on the near
+// field's lose again, when the older kernel's many small CTAs fill the GPU (2
+// columns: 1,352 boxes 36 -> 30, 4,568 boxes 97 -> 109, 5,768 boxes 60 -> 87).
+constexpr int kManyBoxes = 608, kNearMostBoxes = 2432;
 
 // Leaf boxes too few to give every SM two CTAs at one per box and 16 columns.
 bool few_boxes(int64_t boxes, int B) { return boxes * ((B + 15) / 16) < 2 * 152; }
@@ -1466,9 +1468,12 @@ cudaError_t launch_near(const ProductArgs<R> &a, cudaStream_t s, int choice = 0)
     if (choice == 1) return wide_ok ? launch_near_wide<R, 8>(a, s) : cudaErrorInvalidConfiguration;
     if (choice == 2) return wide_ok ? launch_near_wide<R, 16>(a, s) : cudaErrorInvalidConfiguration;
     if (choice == 3) return a.B >= 16 ? launch_near_bt<R, 16>(a, s) : cudaErrorInvalidConfiguration;
-    // register tiles: FP32 from four columns up, from two on trees of many boxes; FP64, which its arithmetic bounds, where the tree has too few
-    // leaf boxes to fill the GPU with one CTA per box (near_tile.cu has the figures of both sides)
-    if (sizeof(R) == 4 ? (a.B >= 4 || (a.B >= 2 && a.nr.nleaf >= kManyBoxes)) : (a.B >= 4 && few_boxes(a.nr.nleaf, a.B))) {
+    // register tiles: FP32 from four columns up, from two on trees of many boxes; FP64, which its arithmetic bounds, where
+    // the tree has too few leaf boxes to fill the GPU with one CTA per box (near_tile.cu has the figures of both sides),
+    // half of that for four columns, which the older kernel takes in one chunk (296 boxes 60 us, 83 by the tile; 64 boxes 83
+    // and 71)
+    if (sizeof(R) == 4 ? (a.B >= 4 || (a.B >= 2 && a.nr.nleaf >= kManyBoxes && a.nr.nleaf < kNearMostBoxes))
+                       : (a.B >= 4 && few_boxes(a.nr.nleaf, a.B) && (a.B > 4 || a.nr.nleaf < 152))) {
         const cudaError_t e = launch_near_tile<R>(a, s);
         if (e != cudaErrorInvalidConfiguration) return e;
     }
