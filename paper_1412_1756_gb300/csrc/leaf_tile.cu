@@ -523,16 +523,15 @@ cudaError_t receive_go(const ProductArgs<R> &a, int Bs, int ncp, cudaStream_t s)
 template <class R>
 cudaError_t launch_radiate_tile(const ProductArgs<R> &a, int Bs, cudaStream_t s)
 {
-    if (a.B == 1) return radiate_go<R, 1>(a, Bs, s);
-    if (a.B == 2 || sizeof(R) == 8) return radiate_go<R, 2>(a, Bs, s);
-    if constexpr (sizeof(R) == 4) return radiate_go<R, 4>(a, Bs, s);
-    return cudaErrorInvalidConfiguration;
+    if (a.B < 2) return cudaErrorInvalidConfiguration;
+    if constexpr (sizeof(R) == 4) return a.B == 2 ? radiate_go<R, 2>(a, Bs, s) : radiate_go<R, 4>(a, Bs, s);
+    else return radiate_go<R, 2>(a, Bs, s);
 }
 
 template <class R>
 cudaError_t launch_receive_tile(const ProductArgs<R> &a, int Bs, cudaStream_t s)
 {
-    if (a.B == 1) return receive_go<R, 1, 16, 1>(a, Bs, 1, s);
+    if (a.B < 2) return cudaErrorInvalidConfiguration;
     const int ncp = (a.B + 1) / 2;
     if constexpr (sizeof(R) == 4) {
         if (ncp <= 4) return receive_go<R, 2, 32, 1>(a, Bs, ncp, s);
@@ -558,8 +557,8 @@ cudaError_t prime_leaf_tile()
 {
     cudaError_t e;
 #define ALLOW(k) do { if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kLeafSmem)) != cudaSuccess) return e; } while (0)
-    ALLOW((k_radiate_tile<R, 1>)); ALLOW((k_radiate_tile<R, 2>));
-    ALLOW((k_receive_tile<R, 1, 16, 1, 1>)); ALLOW((k_receive_tile<R, 2, 16, 1, 1>));
+    ALLOW((k_radiate_tile<R, 2>));
+    ALLOW((k_receive_tile<R, 2, 16, 1, 1>));
     if constexpr (sizeof(R) == 4) {
         ALLOW((k_radiate_tile<R, 4>));
         ALLOW((k_receive_tile<R, 2, 32, 1, 1>)); ALLOW((k_receive_tile<R, 2, 8, 4, 2>));

@@ -245,10 +245,8 @@ cudaError_t go(const ProductArgs<R> &a, int most, cudaStream_t s)
 template <class R>
 cudaError_t launch_near_tile(const ProductArgs<R> &a, cudaStream_t s)
 {
-    if (a.B < 1 || a.nr.nleaf < 1) return cudaErrorInvalidConfiguration;
-    if (a.B == 1) return go<R, 1>(a, 1, s);
-    if (a.B == 2) return go<R, 2>(a, 2, s);
-    if constexpr (sizeof(R) == 4) return go<R, 4>(a, 64, s);
+    if (a.B < 2 || a.nr.nleaf < 1) return cudaErrorInvalidConfiguration;
+    if constexpr (sizeof(R) == 4) return a.B == 2 ? go<R, 2>(a, 2, s) : go<R, 4>(a, 64, s);
     else return go<R, 2>(a, 16, s);
 }
 
@@ -257,7 +255,6 @@ cudaError_t prime_near_tile()
 {
     cudaError_t e;
 #define ALLOW(k) do { if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kNearTileSmem)) != cudaSuccess) return e; } while (0)
-    ALLOW((k_near_tile<R, 1>));
     ALLOW((k_near_tile<R, 2>));
     if constexpr (sizeof(R) == 4) ALLOW((k_near_tile<R, 4>));
 #undef ALLOW

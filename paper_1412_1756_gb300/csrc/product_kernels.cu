@@ -1611,7 +1611,6 @@ cudaError_t launch_receive(const ProductArgs<R> &a, int Bs, cudaStream_t s, int 
     if (choice == 1) return a.B >= 32 ? launch_receive_tiled<R, 32>(a, Bs, s) : cudaErrorInvalidConfiguration;
     if (choice == 2) return a.B >= 16 ? launch_receive_tiled<R, 16>(a, Bs, s) : cudaErrorInvalidConfiguration;
     if (choice == 3) return a.B >= 8 ? launch_receive_tiled<R, 8>(a, Bs, s) : cudaErrorInvalidConfiguration;
-    if (a.B >= 32 && sizeof(R) == 4) return launch_receive_tiled<R, 32>(a, Bs, s);
     if (a.B >= 16) return launch_receive_tiled<R, 16>(a, Bs, s);
     if (a.B >= 8) return launch_receive_tiled<R, 8>(a, Bs, s);
     const int K = a.lv[a.leaf].K;

@@ -457,8 +457,8 @@ __global__ void __launch_bounds__(256, MINB) k_down_win_pp(DevLevel<float> P, De
 // * gam(theta), and gam commutes with the phi interpolation, so the first
 // child's T is scaled by its gam, the second's is scaled and added, and the
 // phi step of the sum is accumulated with the pair's common shift_xy.
-template <int NB, int MINB, bool PAIR = false, int NT = 256>
-__global__ void __launch_bounds__(NT, MINB) k_up_win(DevLevel<float> P, DevLevel<float> Ch, int B, int RS, int Bs,
+template <int NB, int MINB, bool PAIR = false>
+__global__ void __launch_bounds__(256, MINB) k_up_win(DevLevel<float> P, DevLevel<float> Ch, int B, int RS, int Bs,
                                                       int accumulate)
 {
     constexpr int NCP = NB / 2, RL = 32 / NCP, ES = NB / 2;
@@ -663,7 +663,7 @@ cudaError_t down_win_pp_nb(const DevLevel<float> &P, const DevLevel<float> &Ch, 
     return cudaGetLastError();
 }
 
-template <int NB, int MINB, bool PAIR = false, int NT = 256>
+template <int NB, int MINB, bool PAIR = false>
 cudaError_t up_win_nb(const DevLevel<float> &P, const DevLevel<float> &Ch, int B, int Bs, int acc, cudaStream_t s)
 {
     if (PAIR && (!P.shift_xy || !P.gam)) return cudaErrorInvalidConfiguration;
@@ -677,7 +677,7 @@ cudaError_t up_win_nb(const DevLevel<float> &P, const DevLevel<float> &Ch, int B
     const size_t smem = up_win_smem(P, Ch, NB, RS);
     if (smem > kWinSmemCap) return cudaErrorInvalidConfiguration;
     dim3 grid(P.nbox * ((B + NB - 1) / NB) * RS, 2);
-    k_up_win<NB, MINB, PAIR, NT><<<grid, NT, smem, s>>>(P, Ch, B, RS, Bs, acc);
+    k_up_win<NB, MINB, PAIR><<<grid, 256, smem, s>>>(P, Ch, B, RS, Bs, acc);
     return cudaGetLastError();
 }
 
