@@ -217,15 +217,6 @@ __device__ __forceinline__ void stage_field(float *raw, const float *src, int K,
     }
 }
 
-// Two warpgroups per CTA: staging the operands and reading the results back
-// bound these kernels (the tensor pipe is active 1-2 % of the time), and
-// where shared memory leaves room for one or two CTAs per SM the copies are
-// shared out over twice the warps - both groups reach the same tensor-memory
-// lanes and split the columns, tiles or K blocks.  3xTF32, one -> two
-// warpgroups (us): 10,680 unknowns, 16 columns, down 236 -> 148 and 252 ->
-// 166, up 90 -> 68 and 100 -> 88; 28,800 unknowns, 64 columns, down from
-// level 2 2,151 -> 1,294.  Up levels whose CTAs fit three to an SM keep one
-// (28,800 unknowns, up into level 3 947 against 1,039).
 // The tensor-memory allocation, operand images and the shared A tile buffer
 // (steps 1 and 2 never hold it at the same time).
 struct Ctx {
@@ -307,6 +298,18 @@ __device__ __forceinline__ void sync_tmem()
     __syncthreads();
     fence_after();
 }
+
+// Two warpgroups per CTA: staging the operands and reading the results back
+// bound these kernels (the tensor pipe is active 1-2 % of the time), and
+// where an SM has room for one or two CTAs the copies are shared out over
+// twice the warps - both groups reach the same tensor-memory lanes and split
+// the columns, tiles or K blocks.  One -> two warpgroups (us): 3xTF32, 10,680
+// unknowns, 16 columns, down 236 -> 145 and 252 -> 166, up 90 -> 68 and 100 ->
+// 88; 28,800 unknowns, 64 columns, down from level 2 2,151 -> 1,294.  The down
+// pass gains at every level (7,680 unknowns, 14 x 28 samples, 16 columns 127
+// -> 113).  Up levels whose CTAs fit three to an SM keep one (TF32, 28,800
+// unknowns, 64 columns: into 14 x 28 samples 664 against 881; into 21 x 42,
+// whose 256 tensor-memory columns a CTA leave room for two, 365 against 317).
 
 // ------------------------------------------------------------------- up ---
 // grid (parent box, component, column-chunk group); NT threads.  The work
@@ -628,7 +631,10 @@ cudaError_t launch_up_umma(const DevLevel<float> &P, const DevLevel<float> &Ch, 
         kernel<<<grid, threads, smem, s>>>(P, Ch, B, Bs, acc, cpc);
         return cudaGetLastError();
     };
-    if (smem <= (size_t)74 * 1024) return split ? go(k_up_umma<true, 128>, 128) : go(k_up_umma<false, 128>, 128);   // three CTAs per SM
+    // one warpgroup where three CTAs fit an SM: its shared memory and its 512 tensor-memory columns
+    const int ncols = tmem_cols((Ch.nth + 15) / 16 * P.um_up1.N + P.um_up2.N + (P.nph + 15) / 16 * P.um_up2.N);
+    if (smem <= (size_t)74 * 1024 && 3 * ncols <= 512)
+        return split ? go(k_up_umma<true, 128>, 128) : go(k_up_umma<false, 128>, 128);
     return split ? go(k_up_umma<true, 256>, 256) : go(k_up_umma<false, 256>, 256);
 }
 
