@@ -27,12 +27,15 @@
 // columns (below 16) the threads left over after the tiles split the samples
 // (KS ways) and the partial sums are added in a fixed order; otherwise every
 // sum runs over the samples in order.  In FP32 the samples of a tile (two
-// samples with 16 columns and more) are added up first and then join the
-// running sum: chained into it, four roundings per sample are of the running
-// sum's size, and five digits magnify them 700-fold (30,720-unknown sphere,
-// error against FP64 4.7e-5 at 8 columns, 6.8e-5 at 15, 4.5e-5 at 17; so
-// 3.6e-5, 3.9e-5, 3.5e-5, where k_receive_tiled with one rounding per sample
-// has 3.6e-5; reception takes 0-8 % longer).  The field tile is requested one tile
+// samples from 17 to 31 columns) are added up first and then join the running
+// sum: chained into it, four roundings per sample are of the running sum's
+// size, and five digits magnify them 700-fold (30,720-unknown sphere, error
+// against FP64 4.7e-5 at 8 columns, 6.8e-5 at 15, 4.5e-5 at 17; so 3.6e-5,
+// 3.9e-5, 3.5e-5, where k_receive_tiled with one rounding per sample has
+// 3.6e-5; reception takes 0-8 % longer).  From 32 columns up the sum is
+// chained as in k_receive_pairs, which these widths may take as well: any
+// other order would move five-digit products by 1e-4.
+// The field tile is requested one tile
 // ahead and scaled by w_q on its way to shared memory, the patterns arrive
 // by cp.async one tile ahead.  Bound: instruction issue.  Measured, before ->
 // this (FP32, us): 30,720-unknown sphere 2 columns 47 -> 35, 10 columns 117
@@ -226,7 +229,7 @@ template <class R, int CW> struct alignas(CW * 2 * sizeof(R) >= 16 ? 16 : CW * 2
 // ncp column groups (CW columns each) per CTA, CPT of them per thread (group
 // cp, cp + ncp / CPT, ...), tiles of QT samples, RP rows per pass at most;
 // NE: field elements a thread stages per tile.
-template <class R, int CW, int QT, int NE, int CPT>
+template <class R, int CW, int QT, int NE, int CPT, bool SUM>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 && CPT == 1 ? 3 : (sizeof(R) == 4 ? 2 : 1)) k_receive_tile(const int32_t *__restrict__ box_ptr, const Four<R> *__restrict__ V4,
                                                       DevLevel<R> lf, typename Cplx<R>::T *__restrict__ yp, int B, int Bs,
                                                       int ncp, int RP)
@@ -234,7 +237,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && CPT == 1 ? 3 : (sizeof(
     using C = typename Cplx<R>::T;
     using G1 = Cols<R, CW>;
     // acc is one tile's sum, tot the running sum
-    constexpr bool TS = sizeof(R) == 4 && CPT == 1;
+    constexpr bool TS = SUM && CPT == 1;
     constexpr int VP = QT + 1;   // pitch of a staged pattern row: the rows a warp reads fall in different banks
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int GT = 2 * QT * ncp;                            // field tile: [component][sample][column group]
@@ -329,17 +332,25 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && CPT == 1 ? 3 : (sizeof(
             if (ks < KS) {
                 const G1 *gs = Gs + (size_t)buf * GT + cp, *gs2 = gs + QT * ncp;
                 const Four<R> *vs = Vs + (size_t)buf * RP * VP + rg * VP;   // rows past the last: stale values, dropped
-                if constexpr (CPT == 1) {
+                if constexpr (CPT == 1 || !SUM) {
 #pragma unroll 2
                     for (int qx = ks; qx < nq; qx += KS) {
-                        const G1 g0 = gs[qx * ncp], g1 = gs2[qx * ncp];
+                        G1 g0[CPT], g1[CPT];
+#pragma unroll
+                        for (int u = 0; u < CPT; ++u) {
+                            g0[u] = gs[qx * ncp + u * nct];
+                            g1[u] = gs2[qx * ncp + u * nct];
+                        }
 #pragma unroll
                         for (int k = 0; k < kRows; ++k) {
                             const Four<R> v = vs[k * nrg * VP + qx];
 #pragma unroll
-                            for (int c = 0; c < CW; ++c) cmacc(acc[0][k][c], v.x, v.y, g0.v[2 * c], g0.v[2 * c + 1]);
+                            for (int u = 0; u < CPT; ++u) {
 #pragma unroll
-                            for (int c = 0; c < CW; ++c) cmacc(acc[0][k][c], v.z, v.w, g1.v[2 * c], g1.v[2 * c + 1]);
+                                for (int c = 0; c < CW; ++c) cmacc(acc[u][k][c], v.x, v.y, g0[u].v[2 * c], g0[u].v[2 * c + 1]);
+#pragma unroll
+                                for (int c = 0; c < CW; ++c) cmacc(acc[u][k][c], v.z, v.w, g1[u].v[2 * c], g1[u].v[2 * c + 1]);
+                            }
                         }
                     }
                     if (TS) {
@@ -492,7 +503,7 @@ int usual_groups(const ProductArgs<R> &a, int nbox)
     return (mean + mean / 4 + kRows - 1) / kRows;
 }
 
-template <class R, int CW, int QT, int NE, int CPT = 1>
+template <class R, int CW, int QT, int NE, int CPT = 1, bool SUM = sizeof(R) == 4>
 cudaError_t receive_go(const ProductArgs<R> &a, int Bs, int ncp, cudaStream_t s)
 {
     const DevLevel<R> &Lf = a.lv[a.leaf];
@@ -513,7 +524,7 @@ cudaError_t receive_go(const ProductArgs<R> &a, int Bs, int ncp, cudaStream_t s)
     const size_t part = split ? (size_t)256 * kRows * CW * 2 * sizeof(R) : 0;
     const size_t smem = std::max(stage, part);
     if (smem > (size_t)kLeafSmem) return cudaErrorInvalidConfiguration;
-    k_receive_tile<R, CW, QT, NE, CPT><<<dim3((unsigned)ctas, rs), threads, smem, s>>>(
+    k_receive_tile<R, CW, QT, NE, CPT, SUM><<<dim3((unsigned)ctas, rs), threads, smem, s>>>(
         a.nr.box_ptr, reinterpret_cast<const Four<R> *>(a.V), Lf, reinterpret_cast<typename Cplx<R>::T *>(a.yp), a.B, Bs, ncp, RP);
     return cudaGetLastError();
 }
@@ -546,7 +557,8 @@ cudaError_t launch_receive_tile(const ProductArgs<R> &a, int Bs, cudaStream_t s)
         const bool passes = (a.nr.max_rows + kRows - 1) / kRows > std::max(64, (nct * usual_groups(a, a.lv[a.leaf].nbox) + 31) / 32 * 32) / nct;
         const bool full = a.B == 32 || ((rest == 0 || rest > 60) && a.lv[a.leaf].nbox < 4096);
         if ((a.B > 64 && rest > 0 && rest <= 32 && a.nr.max_rows < 96) || (full && passes)) return launch_receive_pairs(a, Bs, 32, s);
-        return receive_go<R, 2, 8, 4, 2>(a, Bs, std::min((ncp + 1) / 2 * 2, 32), s);
+        const int pairs = std::min((ncp + 1) / 2 * 2, 32);
+        return a.B < 32 ? receive_go<R, 2, 8, 4, 2, true>(a, Bs, pairs, s) : receive_go<R, 2, 8, 4, 2, false>(a, Bs, pairs, s);
     } else {
         return receive_go<R, 2, 16, 1>(a, Bs, std::min(ncp, 8), s);
     }
@@ -558,10 +570,10 @@ cudaError_t prime_leaf_tile()
     cudaError_t e;
 #define ALLOW(k) do { if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kLeafSmem)) != cudaSuccess) return e; } while (0)
     ALLOW((k_radiate_tile<R, 2>));
-    ALLOW((k_receive_tile<R, 2, 16, 1, 1>));
+    ALLOW((k_receive_tile<R, 2, 16, 1, 1, sizeof(R) == 4>));
     if constexpr (sizeof(R) == 4) {
         ALLOW((k_radiate_tile<R, 4>));
-        ALLOW((k_receive_tile<R, 2, 32, 1, 1>)); ALLOW((k_receive_tile<R, 2, 8, 4, 2>));
+        ALLOW((k_receive_tile<R, 2, 32, 1, 1, true>)); ALLOW((k_receive_tile<R, 2, 8, 4, 2, true>)); ALLOW((k_receive_tile<R, 2, 8, 4, 2, false>));
     }
 #undef ALLOW
     return cudaSuccess;

@@ -1598,9 +1598,10 @@ cudaError_t launch_receive(const ProductArgs<R> &a, int Bs, cudaStream_t s, int 
         // chunks of four in k_receive (28,800 unknowns, 596 us for four columns, 1,420 for seven by the tile).  Boxes of
         // fewer than 16 rows leave most of a tile's threads idle: only 2-15 columns in FP32 and 8-10 in FP64, where the
         // threads just cover a tile's samples (480 unknowns, us: FP32 32 columns 24 older, 37 tile; FP64 4 columns 31 and 43,
-        // 8 columns 74 and 47, 12 columns 74 and 98).
-        const bool small = a.nr.max_rows < 16, few = few_boxes(a.lv[a.leaf].nbox, a.B);
-        if (sizeof(R) == 8 ? (small ? a.B >= 8 && a.B <= 10 : few ? a.B >= 3 : a.B >= 5 && a.B != 7)
+        // 8 columns 74 and 47, 12 columns 74 and 98).  Trees of fewer than 2,432 unknowns, 16 per SM, keep the 16-column
+        // kernel at 17-31 columns (1,920 unknowns 33 and 39; 3,605 unknowns 94 and 74).
+        const bool small = a.nr.max_rows < 16 || (a.n < 16 * 152 && a.B > 16 && a.B < 32), few = few_boxes(a.lv[a.leaf].nbox, a.B);
+        if (sizeof(R) == 8 ? (a.nr.max_rows < 16 ? a.B >= 8 && a.B <= 10 : few ? a.B >= 3 : a.B >= 5 && a.B != 7)
                            : (a.B >= 2 && (small ? a.B < 16 : a.B != 16))) {
             const cudaError_t e = launch_receive_tile<R>(a, Bs, s);
             if (e != cudaErrorInvalidConfiguration) return e;
