@@ -12,13 +12,14 @@
 // step (RR unknowns x the CTA's samples) ahead, one barrier per step.
 //
 // Measured, the kernels of fixed column chunks before -> this (FP32, us):
-// 30,720-unknown sphere 2 columns 38 -> 29, 10 columns 120 -> 53, 40 columns
-// 115 -> 101; 122,880 unknowns, 34 columns 400 -> 338.  Whole chunks of 64
-// columns stay with k_radiate_quads (618 against 675 on the 115,200-unknown
-// cube), one column with k_radiate (7 against 8 on 480 unknowns).  FP64 is
-// bound by its arithmetic: the tiles win where sample splits spread few boxes
-// over the GPU (1,920 unknowns, 8 columns 77 -> 42) and lose elsewhere
-// (28,800 unknowns, 4 columns 300 -> 500).
+// 30,720-unknown sphere 2 columns 38 -> 29, 10 columns 117 -> 52, 40 columns
+// 115 -> 92; 115,200-unknown cube, five digits, 6 columns 309 -> 199, 80
+// columns 1,107 -> 955.  Whole chunks of 64 columns stay with
+// k_radiate_quads (618 against 675 on the 115,200-unknown cube), one column
+// with k_radiate (7 against 8 on 480 unknowns).  FP64 is bound by its
+// arithmetic: the tiles win where sample splits spread few boxes over the GPU
+// (1,920 unknowns, 8 columns 77 -> 42) and lose elsewhere (28,800 unknowns, 4
+// columns 300 -> 500).
 //
 // Reception: one CTA per (leaf box, column chunk, row split); a thread keeps
 // 4 rows x 2 or 4 columns (the second pair half the chunk away, so that
@@ -39,12 +40,11 @@
 // ahead and scaled by w_q on its way to shared memory, the patterns arrive
 // by cp.async one tile ahead.  Bound: instruction issue.  Measured, before ->
 // this (FP32, us): 30,720-unknown sphere 2 columns 47 -> 35, 10 columns 117
-// -> 59, 40 columns 250 -> 192; 122,880 unknowns, 34 columns 818 -> 537;
-// 115,200-unknown cube, 64 columns 1,307 -> 1,230.  One column (35 against 61
-// on 28,800 unknowns) and exactly 16 (61 against 76 on 10,824) stay with the
-// older kernels.  FP64, 1,920 unknowns, 8 columns 186 -> 80; up to four
-// columns k_receive wins unless boxes are few (28,800 unknowns, 2 columns 325
-// against 440).
+// -> 63, 40 columns 250 -> 193; 122,880 unknowns, 34 columns 818 -> 537;
+// 115,200-unknown cube, 64 columns 1,307 -> 1,230.  FP64: 1,920 unknowns, 8
+// columns 186 -> 80, 32 columns 328 -> 213; 28,800 unknowns, five digits, 32
+// columns 5,244 -> 4,640.  Which widths and trees keep other kernels stands at
+// the rules (launch_receive, launch_receive_tile).
 #include "device.h"
 
 #include <algorithm>

@@ -7,22 +7,22 @@
 // keeps 4 rows x CT columns in registers, so one strip value feeds 2 CT
 // multiply-adds and one x value eight; the threads left over after
 // (rows / 4) x (columns / CT) tiles split the strip columns among
-// themselves, which keeps the CTA full from one right-hand side (36 ways on a
-// 26-row box) to 64 (2 ways).  Chunks of KC strip columns - their values,
+// themselves, which keeps the CTA full from two right-hand sides (36 ways on
+// a 26-row box) to 64 (2 ways).  Chunks of KC strip columns - their values,
 // contiguous in the column-major strip, and the gathered x rows - are staged
 // in shared memory by cp.async one chunk ahead.  The partial sums are added
 // in a fixed order through shared memory at the end.
 //
-// Bound: instruction issue (69 % active at 64 columns); with one or two
-// columns the bytes of the strips.  Measured, one row per thread and chunks
-// of 16 columns before -> this (FP32, us): 30,720-unknown sphere 2 columns 44
-// -> 40, 10 columns 120 -> 67, 40 columns 245 -> 132; 122,880 unknowns, 34
-// columns 765 -> 400; 115,200-unknown cube, 64 columns 313 -> 293.  One
-// column is left to the kernel of one row per thread (28 against 30 us on
-// 28,800 unknowns).  FP64 is bound by its arithmetic (two multiply-adds per
-// SM and cycle): the tiles win only where row splits spread few boxes over
-// the GPU (1,920 unknowns, 8 columns 105 -> 73) and lose elsewhere (28,800
-// unknowns, 4 columns 134 -> 185).
+// Bound: instruction issue (69 % active at 64 columns); with two columns the
+// bytes of the strips.  Measured, one row per thread and chunks of 16 columns
+// before -> this (FP32, us): 30,720-unknown sphere 2 columns 44 -> 36, 10
+// columns 120 -> 67, 40 columns 245 -> 132; 122,880 unknowns, 34 columns 765
+// -> 400; 115,200-unknown cube, 64 columns 313 -> 293.  One column is left to
+// the kernel of one row per thread (28 against 30 us on 28,800 unknowns).
+// FP64 is bound by its arithmetic (two multiply-adds per SM and cycle): the
+// tiles win only where row splits spread few boxes over the GPU (1,920
+// unknowns, 8 columns 105 -> 73) and lose elsewhere (28,800 unknowns, 4
+// columns 134 -> 185).
 #include "device.h"
 
 #include <algorithm>

@@ -1103,10 +1103,11 @@ __device__ __forceinline__ void sample_acc(C &acc, const C4 &v, const C &g0, con
 // block, scaled by the weights, in shared memory; a warp takes two unknowns at
 // a time, lanes split into LB column lanes x 32/LB sample lanes, reduced with
 // shuffles (the first step leaves each half of the lanes one unknown).  FP64
-// is bound by its arithmetic, so what counts is operations: weights per
-// sample and unknown and five shuffle steps per unknown had made 100 of the
-// 72 that one unknown's 288 samples need (28,800 unknowns, 1 column, 224 us;
-// now 162.  2 columns 416 -> 325).
+// is bound by its arithmetic, so what counts is operations.  One unknown, one
+// column and 288 samples (nine a lane, two components) need 72 multiply-adds
+// a lane; weights applied to each unknown's sum (two a sample, 18) and five
+// shuffle steps of two additions made that 100, now 77 (28,800 unknowns, 1
+// column 221 -> 166 us, 2 columns 400 -> 313).
 template <class R, int LB>
 __global__ void __launch_bounds__(256) k_receive(const int32_t *__restrict__ box_ptr,
                                                  const typename Cx<R>::T4 *__restrict__ V4, DevLevel<R> lf,
