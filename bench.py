@@ -175,11 +175,12 @@ def kernel_digest():
     return h.hexdigest()[:16]
 
 
-# DRAM bytes (read + write) per launch of the dominant stage measured by ncu
+# DRAM bytes (read + write) per launch of the dominant stages measured by ncu
 # at B = 64: {(workload, stage, kernel source digest): bytes}.  Summaries in
-# profiles/ (k_translate_q4_cube8m-6lv_B64.md).
+# profiles/ (dram_cube8m-6lv_B64.md).
 NCU_TRAFFIC = {
-    ("cube8m-6lv", "translate5", "d39c757f68fed696"): 1_764_666_000 + 1_665_967_000,
+    ("cube8m-6lv", "down4", "977a6dd3763107d3"): 2_410_574_080 + 1_647_474_176,
+    ("cube8m-6lv", "translate5", "977a6dd3763107d3"): 1_764_869_120 + 1_667_068_672,
 }
 
 
